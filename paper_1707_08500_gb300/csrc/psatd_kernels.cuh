@@ -34,6 +34,9 @@
 #ifndef PSATD_MINB_A
 #define PSATD_MINB_A 5
 #endif
+#ifndef PSATD_MINB_HEAT
+#define PSATD_MINB_HEAT 4 // 64 registers; 0.48 ms at 2, 0.37 at 3, 0.33 at 4 on 64 boxes of 96^3
+#endif
 #ifndef PSATD_MINB_A_FIXED
 #define PSATD_MINB_A_FIXED 6    // compile-time geometry: fewer registers live, one more CTA fits
 #endif
@@ -46,49 +49,33 @@
 
 namespace psatd {
 
+template <typename T> struct vec2;
+template <> struct vec2<float> { using type = float2; };
+template <> struct vec2<double> { using type = double2; };
+
 // A table twiddle as an FP32 hi + lo pair (lo = 0 in FP64).
 template <typename T>
 struct alignas(4 * sizeof(T)) twd { cpx<T> hi, lo; };
 
-// FP32 table twiddles: the hi part alone (PSATD_TW_HILO 0, the default),
-// which the host rounds so that each twiddle's magnitude is as close to 1 as
-// neighbouring FP32 values allow (the transform then stays closer to
-// unitary; the phase error this trades in cancels between a forward
-// transform and its inverse), or hi + lo pairs (PSATD_TW_HILO 1, FP64-exact
-// twiddles at twice the multiply cost).  Measured over 100 FP32 steps
-// against the FP64 oracle: 5.1e-6 (hi alone) and 3.8e-6 (hi + lo).
-#ifndef PSATD_TW_HILO
-#define PSATD_TW_HILO 0
-#endif
-
+// The kernels use the hi part alone, which the host rounds so that each FP32
+// twiddle's magnitude is as close to 1 as neighbouring values allow (the
+// transform then stays closer to unitary; the phase error this trades in
+// cancels between a forward transform and its inverse).  Measured over 100
+// FP32 steps against the FP64 oracle: 5.1e-6, and 3.8e-6 with hi + lo
+// products, at twice their cost.
 template <typename T>
 __device__ __forceinline__ twd<T> ld_tw(const twd<T>* p) {
+    using V = typename vec2<T>::type;
+    const V v = __ldg(reinterpret_cast<const V*>(p));
     twd<T> t;
-    if constexpr (sizeof(T) == 4 && !PSATD_TW_HILO) {
-        const float2 v = __ldg(reinterpret_cast<const float2*>(p));
-        t.hi = mk(v.x, v.y);
-        t.lo = mk(0.f, 0.f);
-    } else if constexpr (sizeof(T) == 4) {
-        const float4 v = __ldg(reinterpret_cast<const float4*>(p));
-        t.hi = mk(v.x, v.y);
-        t.lo = mk(v.z, v.w);
-    } else {
-        const double2 v = __ldg(reinterpret_cast<const double2*>(p));
-        t.hi = mk(v.x, v.y);
-        t.lo = mk(0.0, 0.0);
-    }
+    t.hi = mk(v.x, v.y);
+    t.lo = mk(T(0), T(0));
     return t;
 }
 template <typename T>   // v * w
-__device__ __forceinline__ cpx<T> mul_tw(cpx<T> v, const twd<T>& w) {
-    if constexpr (sizeof(T) == 4 && !PSATD_TW_HILO) return cmul(v, w.hi);
-    else return cmul_const(v, w.hi.x, w.lo.x, w.hi.y, w.lo.y);
-}
+__device__ __forceinline__ cpx<T> mul_tw(cpx<T> v, const twd<T>& w) { return cmul(v, w.hi); }
 template <typename T>   // v * conj(w)
-__device__ __forceinline__ cpx<T> mul_tw_conj(cpx<T> v, const twd<T>& w) {
-    if constexpr (sizeof(T) == 4 && !PSATD_TW_HILO) return cmulc(v, w.hi);
-    else return cmul_const(v, w.hi.x, w.lo.x, -w.hi.y, -w.lo.y);
-}
+__device__ __forceinline__ cpx<T> mul_tw_conj(cpx<T> v, const twd<T>& w) { return cmulc(v, w.hi); }
 
 template <typename T>
 struct Args {
@@ -115,9 +102,6 @@ struct Args {
 
 
 
-template <typename T> struct vec2;
-template <> struct vec2<float> { using type = float2; };
-template <> struct vec2<double> { using type = double2; };
 template <typename T>
 __device__ __forceinline__ cpx<T> ldg_c(const cpx<T>* p) {
     const auto v = __ldg(reinterpret_cast<const typename vec2<T>::type*>(p));
@@ -847,7 +831,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? PSATD_MINB_B : 2) k
 // B = (1 - exp(-x))/x, x = D dt |[k]|^2 (both scaled by 1/(Lx Ly Lz)), read
 // from the first two coefficient arrays; S is the optional source (field 1).
 template <typename T>
-__global__ void __launch_bounds__(kThreads) k_pass_b_heat(Args<T> a) {
+__global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? PSATD_MINB_HEAT : 2) k_pass_b_heat(Args<T> a) {
     extern __shared__ __align__(16) unsigned char smraw[];
     cpx<T>* sm = reinterpret_cast<cpx<T>*>(smraw);
     __shared__ SubDesc d;

@@ -21,11 +21,11 @@ struct alignas(2 * sizeof(T)) cpx {
     T x, y;
 };
 
-// Two FP32 lanes advanced by one packed instruction (FFMA2 / FMUL2 of the
-// sm_100 family): the same operation on two independent data sets, e.g. two
-// columns that share every constant and twiddle.  Additions are issued as
-// fused multiply-adds with a unit factor, which round exactly like an
-// addition.
+// Two FP32 lanes advanced by one packed instruction (FFMA2 / FMUL2 / FADD2 of
+// the sm_100 family): the same operation on two independent data sets, e.g. two
+// columns that share every constant and twiddle.  Measured on this part: a
+// packed instruction takes the pipe for two of its cycles (the same FP32 rate
+// as scalar code) but one issue slot, and negating an operand is free.
 struct __align__(8) P2 {
     float x, y;   // lane 0, lane 1
     P2() = default;
@@ -38,9 +38,9 @@ __device__ __forceinline__ float fma_t(float a, float b, float c) { return __fma
 __device__ __forceinline__ double fma_t(double a, double b, double c) { return __fma_rn(a, b, c); }
 __device__ __forceinline__ P2 fma_t(P2 a, P2 b, P2 c) { return p2of(__ffma2_rn(f2of(a), f2of(b), f2of(c))); }
 __device__ __forceinline__ P2 operator*(P2 a, P2 b) { return p2of(__fmul2_rn(f2of(a), f2of(b))); }
-__device__ __forceinline__ P2 operator+(P2 a, P2 b) { return fma_t(a, P2(1.f), b); }
-__device__ __forceinline__ P2 operator-(P2 a, P2 b) { return fma_t(b, P2(-1.f), a); }
-__device__ __forceinline__ P2 operator-(P2 a) { return a * P2(-1.f); }
+__device__ __forceinline__ P2 operator-(P2 a) { return P2(-a.x, -a.y); }
+__device__ __forceinline__ P2 operator+(P2 a, P2 b) { return p2of(__fadd2_rn(f2of(a), f2of(b))); }
+__device__ __forceinline__ P2 operator-(P2 a, P2 b) { return p2of(__fadd2_rn(f2of(a), f2of(-b))); }
 __device__ __forceinline__ P2& operator+=(P2& a, P2 b) { a = a + b; return a; }
 
 template <typename T>
@@ -82,17 +82,21 @@ constexpr long quad_of(long m, long N) { return (4 * (((m % N) + N) % N)) / N; }
 constexpr double phi_of(long m, long N) {
     return (kPi / 2) * double(4 * (((m % N) + N) % N) - quad_of(m, N) * N) / double(N);
 }
+// +-1/2 exactly at multiples of 30 degrees (the series ends within an ulp of it)
+constexpr double snap_half(double v) {
+    return v > 0.5 - 1e-15 && v < 0.5 + 1e-15 ? 0.5 : v > -0.5 - 1e-15 && v < -0.5 + 1e-15 ? -0.5 : v;
+}
 constexpr double cos2pi(long m, long N) {
-    return quad_of(m, N) == 0 ? taylor_cos(phi_of(m, N))
-         : quad_of(m, N) == 1 ? -taylor_sin(phi_of(m, N))
-         : quad_of(m, N) == 2 ? -taylor_cos(phi_of(m, N))
-                              : taylor_sin(phi_of(m, N));
+    return snap_half(quad_of(m, N) == 0 ? taylor_cos(phi_of(m, N))
+                   : quad_of(m, N) == 1 ? -taylor_sin(phi_of(m, N))
+                   : quad_of(m, N) == 2 ? -taylor_cos(phi_of(m, N))
+                                        : taylor_sin(phi_of(m, N)));
 }
 constexpr double sin2pi(long m, long N) {
-    return quad_of(m, N) == 0 ? taylor_sin(phi_of(m, N))
-         : quad_of(m, N) == 1 ? taylor_cos(phi_of(m, N))
-         : quad_of(m, N) == 2 ? -taylor_sin(phi_of(m, N))
-                              : -taylor_cos(phi_of(m, N));
+    return snap_half(quad_of(m, N) == 0 ? taylor_sin(phi_of(m, N))
+                   : quad_of(m, N) == 1 ? taylor_cos(phi_of(m, N))
+                   : quad_of(m, N) == 2 ? -taylor_sin(phi_of(m, N))
+                                        : -taylor_cos(phi_of(m, N)));
 }
 
 // ---- compile-time loop ----------------------------------------------------
@@ -129,34 +133,17 @@ template <>
 constexpr P2 hi_of<P2>(double v) { return P2(float(v)); }
 template <>
 constexpr P2 lo_of<P2>(double v) { return P2(float(v - double(float(v)))); }
+// Whether the FP32 constant v needs its lo part (+-1/2 and the like do not).
+template <typename T>
+constexpr bool has_lo(double v) { return Split32<T>::kOn && v - double(float(v)) != 0.0; }
+constexpr double abs_c(double v) { return v < 0 ? -v : v; }
 
-template <typename T>
-constexpr bool kPacked = std::is_same<T, P2>::value;
-
-// v * (c + i s) with c, s given as (hi, lo) pairs; msh, msl = -sh, -sl are
-// passed separately so that packed lanes need no negation instruction (the
-// scalar forms leave the multiply-adds to the compiler)
-template <typename T>
-__device__ __forceinline__ cpx<T> cmul_const4(cpx<T> v, T ch, T cl, T sh, T sl, T msh, T msl) {
-    if constexpr (kPacked<T>) {
-        if constexpr (Split32<T>::kOn) {
-            const T tr = fma_t(v.x, cl, v.y * msl);
-            const T ti = fma_t(v.x, sl, v.y * cl);
-            return mk(fma_t(v.x, ch, fma_t(v.y, msh, tr)), fma_t(v.x, sh, fma_t(v.y, ch, ti)));
-        } else {
-            return mk(fma_t(v.x, ch, v.y * msh), fma_t(v.x, sh, v.y * ch));
-        }
-    } else if constexpr (Split32<T>::kOn) {
-        const T tr = fmaf(v.x, cl, -v.y * sl);
-        const T ti = fmaf(v.x, sl, v.y * cl);
-        return mk(fmaf(v.x, ch, fmaf(-v.y, sh, tr)), fmaf(v.x, sh, fmaf(v.y, ch, ti)));
-    } else {
-        return mk(v.x * ch - v.y * sh, v.x * sh + v.y * ch);
-    }
-}
-template <typename T>
-__device__ __forceinline__ cpx<T> cmul_const(cpx<T> v, T ch, T cl, T sh, T sl) {
-    return cmul_const4(v, ch, cl, sh, sl, T(-sh), T(-sl));
+// Constants are applied by magnitude, so that c and -c share one register; the
+// sign goes to the other operand (free).
+template <bool NEG, typename T>
+__device__ __forceinline__ T sgn(T v) {
+    if constexpr (NEG) return -v;
+    else return v;
 }
 
 // multiply by exp(sgn 2 pi i M / N), sgn = -1 forward, +1 inverse
@@ -174,7 +161,35 @@ __device__ __forceinline__ cpx<T> twiddle(cpx<T> v) {
     } else {
         constexpr double c = cos2pi(m, N);
         constexpr double s = INV ? sin2pi(m, N) : -sin2pi(m, N);
-        return cmul_const4(v, hi_of<T>(c), lo_of<T>(c), hi_of<T>(s), lo_of<T>(s), hi_of<T>(-s), lo_of<T>(-s));
+        if constexpr (!Split32<T>::kOn) {
+            constexpr T cc = T(c), ss = T(s);
+            return mk(v.x * cc - v.y * ss, v.x * ss + v.y * cc);
+        }
+        constexpr double cm = abs_c(c), sm = abs_c(s);
+        // (x c - y s) + i (x s + y c), the lo parts first
+        const T xc = sgn<(c < 0)>(v.x), yc = sgn<(c < 0)>(v.y);
+        const T xs = sgn<(s < 0)>(v.x), ys = sgn<(s > 0)>(v.y);
+        if constexpr (Split32<T>::kOn && 8 * m % N == 0) {   // c = +-s: one product (hi + lo) for each part
+            const T u = xc + ys, w = yc + xs;
+            return mk(fma_t(u, hi_of<T>(cm), u * lo_of<T>(cm)), fma_t(w, hi_of<T>(cm), w * lo_of<T>(cm)));
+        }
+        T re, im;
+        if constexpr (has_lo<T>(cm) && has_lo<T>(sm)) {
+            re = fma_t(xc, lo_of<T>(cm), ys * lo_of<T>(sm));
+            im = fma_t(yc, lo_of<T>(cm), xs * lo_of<T>(sm));
+            re = fma_t(ys, hi_of<T>(sm), re);
+            im = fma_t(xs, hi_of<T>(sm), im);
+        } else if constexpr (has_lo<T>(cm)) {
+            re = fma_t(ys, hi_of<T>(sm), xc * lo_of<T>(cm));
+            im = fma_t(xs, hi_of<T>(sm), yc * lo_of<T>(cm));
+        } else if constexpr (has_lo<T>(sm)) {
+            re = fma_t(ys, hi_of<T>(sm), ys * lo_of<T>(sm));
+            im = fma_t(xs, hi_of<T>(sm), xs * lo_of<T>(sm));
+        } else {
+            re = ys * hi_of<T>(sm);
+            im = xs * hi_of<T>(sm);
+        }
+        return mk(fma_t(xc, hi_of<T>(cm), re), fma_t(yc, hi_of<T>(cm), im));
     }
 }
 
@@ -201,19 +216,13 @@ template <bool INV>
 struct Dft<4, INV> {
     template <typename T>
     __device__ __forceinline__ static void run(cpx<T>* v) {
-        cpx<T> a = v[0] + v[2], b = v[0] - v[2], c = v[1] + v[3], d = v[1] - v[3];
+        const cpx<T> a = v[0] + v[2], b = v[0] - v[2], c = v[1] + v[3], d = v[1] - v[3];
         v[0] = a + c;
         v[2] = a - c;
-        if constexpr (kPacked<T>) {
-            // b -/+ i d, written out so that no component is negated on its own
-            const cpx<T> bm = mk(b.x + d.y, b.y - d.x), bp = mk(b.x - d.y, b.y + d.x);
-            if (INV) { v[1] = bp; v[3] = bm; }
-            else     { v[1] = bm; v[3] = bp; }
-        } else {
-            cpx<T> id = mul_i(d);
-            if (INV) { v[1] = b + id; v[3] = b - id; }
-            else     { v[1] = b - id; v[3] = b + id; }
-        }
+        // b -/+ i d
+        const cpx<T> bm = mk(b.x + d.y, b.y - d.x), bp = mk(b.x - d.y, b.y + d.x);
+        if (INV) { v[1] = bp; v[3] = bm; }
+        else     { v[1] = bm; v[3] = bp; }
     }
 };
 
@@ -234,32 +243,40 @@ struct DftPrime {
         v[0] = s0;
         static_for<H>([&](auto kc) {
             constexpr int k = decltype(kc)::value + 1;
-            cpx<T> R = x0, Q = mk(T(0), T(0));
-            cpx<T> Rl = mk(T(0), T(0)), Ql = mk(T(0), T(0));
+            cpx<T> R = x0, Q;
+            cpx<T> Rl, Ql;                       // lo parts of the constants, summed apart
             static_for<H>([&](auto jc) {
                 constexpr int j = decltype(jc)::value + 1;
-                constexpr double c = cos2pi((long)j * k, P);
-                constexpr double s = sin2pi((long)j * k, P);
-                constexpr T ch = hi_of<T>(c), sh = hi_of<T>(s);
-                if constexpr (kPacked<T>) {     // packed lanes: explicit multiply-adds
-                    R.x = fma_t(a[j - 1].x, ch, R.x); R.y = fma_t(a[j - 1].y, ch, R.y);
-                    Q.x = fma_t(b[j - 1].x, sh, Q.x); Q.y = fma_t(b[j - 1].y, sh, Q.y);
-                } else {
-                    R.x += a[j - 1].x * ch; R.y += a[j - 1].y * ch;
-                    Q.x += b[j - 1].x * sh; Q.y += b[j - 1].y * sh;
+                constexpr double c = cos2pi((long)j * k, P), s = sin2pi((long)j * k, P);
+                if constexpr (!Split32<T>::kOn) {
+                    constexpr T cc = T(c), ss = T(s);
+                    if constexpr (j == 1) Q = mk(T(0), T(0));
+                    R.x += a[j - 1].x * cc; R.y += a[j - 1].y * cc;
+                    Q.x += b[j - 1].x * ss; Q.y += b[j - 1].y * ss;
+                    return;
                 }
-                if constexpr (Split32<T>::kOn) {
-                    constexpr T cl = lo_of<T>(c), sl = lo_of<T>(s);
-                    if constexpr (kPacked<T>) {
-                        Rl.x = fma_t(a[j - 1].x, cl, Rl.x); Rl.y = fma_t(a[j - 1].y, cl, Rl.y);
-                        Ql.x = fma_t(b[j - 1].x, sl, Ql.x); Ql.y = fma_t(b[j - 1].y, sl, Ql.y);
-                    } else {
-                        Rl.x += a[j - 1].x * cl; Rl.y += a[j - 1].y * cl;
-                        Ql.x += b[j - 1].x * sl; Ql.y += b[j - 1].y * sl;
-                    }
+                constexpr double cm = abs_c(c), sm = abs_c(s);
+                const cpx<T> ac = mk(sgn<(c < 0)>(a[j - 1].x), sgn<(c < 0)>(a[j - 1].y));
+                const cpx<T> bs = mk(sgn<(s < 0)>(b[j - 1].x), sgn<(s < 0)>(b[j - 1].y));
+                if constexpr (has_lo<T>(cm)) {
+                    constexpr T cl = lo_of<T>(cm);
+                    if constexpr (j == 1) Rl = mk(ac.x * cl, ac.y * cl);
+                    else Rl = mk(fma_t(ac.x, cl, Rl.x), fma_t(ac.y, cl, Rl.y));
                 }
+                if constexpr (has_lo<T>(sm)) {
+                    constexpr T sl = lo_of<T>(sm);
+                    if constexpr (j == 1) Ql = mk(bs.x * sl, bs.y * sl);
+                    else Ql = mk(fma_t(bs.x, sl, Ql.x), fma_t(bs.y, sl, Ql.y));
+                }
+                constexpr T ch = hi_of<T>(cm), sh = hi_of<T>(sm);
+                R = mk(fma_t(ac.x, ch, R.x), fma_t(ac.y, ch, R.y));
+                // P = 3 has one sine: its lo product starts the sum
+                if constexpr (j == 1 && H == 1 && has_lo<T>(sm)) Q = mk(fma_t(bs.x, sh, Ql.x), fma_t(bs.y, sh, Ql.y));
+                else if constexpr (j == 1) Q = mk(bs.x * sh, bs.y * sh);
+                else Q = mk(fma_t(bs.x, sh, Q.x), fma_t(bs.y, sh, Q.y));
             });
-            if constexpr (Split32<T>::kOn) { R = R + Rl; Q = Q + Ql; }
+            // every constant but the cosine of P = 3 (-1/2) has a lo part
+            if constexpr (Split32<T>::kOn && H > 1) { R = R + Rl; Q = Q + Ql; }
             // X_k = R + sgn i Q, X_{P-k} = R - sgn i Q
             if (INV) { v[k] = mk(R.x - Q.y, R.y + Q.x); v[P - k] = mk(R.x + Q.y, R.y - Q.x); }
             else     { v[k] = mk(R.x + Q.y, R.y - Q.x); v[P - k] = mk(R.x - Q.y, R.y + Q.x); }
