@@ -6,7 +6,6 @@ namespace psatd {
 
 constexpr int kMaxDft = 16;       // largest register DFT
 constexpr int kThreads = 256;     // threads per CTA of every stage kernel
-constexpr int kSegSmem = 64;      // exchange segments staged in shared memory per CTA
 constexpr int kPlaneSmemMax = 216 * 1024;   // dynamic shared memory of one stage tile (the rest: static)
 constexpr int kSplitRowBytes = 32 * 1024;   // row block of the split-plane schedule
 

@@ -37,6 +37,9 @@
 #ifndef PSATD_MINB_HEAT
 #define PSATD_MINB_HEAT 4 // 64 registers; 0.48 ms at 2, 0.37 at 3, 0.33 at 4 on 64 boxes of 96^3
 #endif
+#ifndef PSATD_MINB_ROWS
+#define PSATD_MINB_ROWS 4
+#endif
 #ifndef PSATD_MINB_A_FIXED
 #define PSATD_MINB_A_FIXED 6    // compile-time geometry: fewer registers live, one more CTA fits
 #endif
@@ -124,28 +127,6 @@ __device__ __forceinline__ void stcs_c(cpx<T>* p, cpx<T> v) {
     using V = typename vec2<T>::type;
     V w; w.x = v.x; w.y = v.y;
     __stcs(reinterpret_cast<V*>(p), w);
-}
-
-// Rows [0, ny) of a segment whose row holds a power-of-two number ex4 <= NT
-// of 16-byte pieces (guard images 16 cells wide, valid rows of 64), from
-// shared memory (row stride rs elements) to global memory (row stride dld):
-// each of the NT threads keeps one piece column and steps down the rows by
-// pointer increments, with no division.  Returns false, storing nothing,
-// for other widths.
-template <int NT, typename T>
-__device__ __forceinline__ bool store_rows_pow2(T* dst, int64_t dld, const T* sp, int rs, int ex4, int ny) {
-    if (ex4 <= 0 || (ex4 & (ex4 - 1)) != 0 || ex4 > NT) return false;
-    const int lg = 31 - __clz(ex4), x4 = int(threadIdx.x) & (ex4 - 1);
-    const int y0 = int(threadIdx.x) >> lg, dyy = NT >> lg;
-    const T* s = sp + y0 * rs + 4 * x4;
-    T* o = dst + int64_t(y0) * dld + 4 * x4;
-    const int64_t ostep = int64_t(dyy) * dld;
-    for (int yy = y0; yy < ny; yy += dyy, s += dyy * rs, o += ostep) {
-        const cpx<T> u = *reinterpret_cast<const cpx<T>*>(s);
-        const cpx<T> w = *reinterpret_cast<const cpx<T>*>(s + 2);
-        stcs4(o, cpx4<T>{u.x, u.y, w.x, w.y});
-    }
-    return true;
 }
 
 // ---- asynchronous global -> shared copies (no register staging) ------------
@@ -580,6 +561,109 @@ struct GeoFix {
           az{L, split_first(L), L / split_first(L), d.az.tw, 0, 0} {}
 };
 
+// ---- the store of the inverse stages (guard replacement, Fig. 3 step 3) --------
+// An exchange segment's part of one output plane: `rows` rows of `ex` cells
+// from shared memory (offset sp) to an arena (element offset dst, rows ld
+// apart).  lg: log2 of the row's 16-byte pieces when they are a power of two
+// and both sides are aligned, -1 for other aligned rows, -2 for the rest.
+struct StoreRec { int64_t dst; int sp, ld, ex, rows, lg, pad; };
+constexpr int kStoreRec = 64;
+struct StorePlan { StoreRec rec[kStoreRec]; int n, next; };
+
+// Records of the segments from number g on that hold rows [ya, yb) of plane z
+// of box d (row ya at offset 0 of shared memory when org = ya, rows rs apart),
+// by one warp, a lane per segment: up to kStoreRec of them, and the number of
+// the first segment left.  A plane meets half of a box's 27 segments or so;
+// finding them and their addresses once, beside the copy that the block waits
+// for, and not in every thread, took pass C from 0.650 to 0.546 ms on 64 boxes
+// of 96^3 and from 0.368 to 0.258 ms on 48 uneven boxes.
+template <typename T>
+__device__ __forceinline__ void plan_stores(const Args<T>& a, const SubDesc& d, int g, int z, int ya, int yb, int org, int rs,
+                                            StorePlan* p) {
+    const int lane = int(threadIdx.x) & 31;
+    int n = 0;
+    for (; g < d.seg_end && n + 32 <= kStoreRec; g += 32) {
+        StoreRec r;
+        bool act = false;
+        if (g + lane < d.seg_end) {
+            const Segment& s = a.segs[g + lane];
+            const int y0 = max(s.y0, ya), y1 = min(s.y0 + s.ey, yb);
+            act = z >= s.z0 && z < s.z0 + s.ez && y0 < y1 && (!a.own_only || s.identity);
+            r.dst = s.dst_off + (int64_t(z + s.dz) * s.dLy + y0 + s.dy) * s.dLx + s.x0 + s.dx;
+            r.sp = (y0 - org) * rs + s.x0;
+            r.ld = s.dLx;
+            r.ex = s.ex;
+            r.rows = y1 - y0;
+            const int e4 = s.ex >> 2;
+            r.lg = !s.vec4 ? -2 : (e4 & (e4 - 1)) == 0 && e4 <= 128 ? 31 - __clz(e4) : -1;
+            r.pad = 0;
+        }
+        const unsigned m = __ballot_sync(0xffffffffu, act);
+        if (act) p->rec[n + __popc(m & ((1u << lane) - 1u))] = r;
+        n += __popc(m);
+    }
+    if (lane == 0) {
+        p->n = n;
+        p->next = g;
+    }
+}
+
+// The planned stores, by the NT threads of the block: for a power-of-two
+// number of pieces each thread keeps one piece column and steps down the rows
+// by pointer increments; other widths are flattened over rows and pieces.
+template <int NT, typename T>
+__device__ __forceinline__ void run_stores(const StorePlan& p, T* out, const T* rp, int rs) {
+    static_assert(NT >= 128, "a row of up to 128 pieces per block step");
+    for (int k = 0; k < p.n; ++k) {
+        const StoreRec r = p.rec[k];
+        T* dst = out + r.dst;
+        const T* sp = rp + r.sp;
+        if (r.lg >= 0) {
+            const int x4 = int(threadIdx.x) & ((1 << r.lg) - 1), y0 = int(threadIdx.x) >> r.lg, dy = NT >> r.lg;
+            const T* s = sp + y0 * rs + 4 * x4;
+            T* o = dst + int64_t(y0) * r.ld + 4 * x4;
+            const int64_t ostep = int64_t(dy) * r.ld;
+            for (int y = y0; y < r.rows; y += dy, s += dy * rs, o += ostep) {
+                const cpx<T> u = *reinterpret_cast<const cpx<T>*>(s);
+                const cpx<T> w = *reinterpret_cast<const cpx<T>*>(s + 2);
+                stcs4(o, cpx4<T>{u.x, u.y, w.x, w.y});
+            }
+        } else {
+            const int count = r.lg == -1 ? r.ex >> 2 : r.ex;
+            int y = int(threadIdx.x) / count, x = int(threadIdx.x) - y * count;
+            const int dy = NT / count, dx = NT - dy * count;
+            while (y < r.rows) {
+                if (r.lg == -1) {
+                    const cpx<T> u = *reinterpret_cast<const cpx<T>*>(sp + y * rs + 4 * x);
+                    const cpx<T> w = *reinterpret_cast<const cpx<T>*>(sp + y * rs + 4 * x + 2);
+                    stcs4(dst + int64_t(y) * r.ld + 4 * x, cpx4<T>{u.x, u.y, w.x, w.y});
+                } else {
+                    __stcs(dst + int64_t(y) * r.ld + x, sp[y * rs + x]);
+                }
+                x += dx;
+                y += dy;
+                if (x >= count) { x -= count; ++y; }
+            }
+        }
+    }
+}
+
+// All stores of a plane whose first records are planned; the rest, if any, are
+// planned and run in further rounds (warp `w` plans).  The caller synchronises
+// the block before the plan or the rows change.
+template <int NT, typename T>
+__device__ __forceinline__ void store_plane(const Args<T>& a, const SubDesc& d, int z, int ya, int yb, int org, int rs,
+                                            StorePlan* p, int w, T* out, const T* rp) {
+    for (;;) {
+        run_stores<NT>(*p, out, rp, rs);
+        const int next = p->next;
+        if (next >= d.seg_end) break;
+        __syncthreads();
+        if (int(threadIdx.x) >> 5 == w) plan_stores(a, d, next, z, ya, yb, org, rs, p);
+        __syncthreads();
+    }
+}
+
 // ---- pass A: x (real) and y forward transforms of one plane ---------------
 template <typename T, class G>
 __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? (G::kFixed ? PSATD_MINB_A_FIXED : PSATD_MINB_A) : 2)
@@ -897,7 +981,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? PSATD_MINB_C : 2) k
     extern __shared__ __align__(16) unsigned char smraw[];
     cpx<T>* sm = reinterpret_cast<cpx<T>*>(smraw);
     __shared__ SubDesc d;
-    __shared__ Segment segs[kSegSmem];
+    __shared__ StorePlan plan;
     __shared__ int64_t s_ticket[2];
     Tickets<T> tk(a, s_ticket);
     for (int64_t it = tk.current(); it >= 0; tk.advance(), it = tk.current()) {
@@ -912,13 +996,9 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? PSATD_MINB_C : 2) k
         const int h = g.h, pitch = g.pitch, lxh = g.lxh;
         const cpx<T>* src = a.spec + d.spec_off + int64_t(f * Lz + z) * g.q;
         loop2(lxh, Ly, [&](int y, int c) { cp_async_c(sm + y * pitch + c, src + y * lxh + c); });
-        // this subdomain's exchange segments (the first kSegSmem of them)
-        const int nsg = min(d.seg_end - d.seg_begin, kSegSmem);
-        {
-            const int* gs = reinterpret_cast<const int*>(a.segs + d.seg_begin);
-            int* ss = reinterpret_cast<int*>(segs);
-            for (int i = threadIdx.x; i < nsg * int(sizeof(Segment) / 4); i += kThreads) ss[i] = __ldg(gs + i);
-        }
+        // where this plane's cells go, found while the copy is under way
+        const int rs = 2 * pitch;                         // real row stride
+        if (threadIdx.x >= kThreads - 32) plan_stores(a, d, d.seg_begin, z, 0, Ly, 0, rs, &plan);
         cp_async_wait_all();
         __syncthreads();
         fft_inv<false, T, G::kThree>(sm, g.ay, Batch{lxh, 1, 0, 0, pitch, 1}, a.tw);
@@ -928,25 +1008,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? PSATD_MINB_C : 2) k
         __syncthreads();
         fft_inv<false, T, G::kThree>(rows, g.ax, Batch{ny, pitch, 0, 0, 1, 1}, a.tw);
         // store the valid cells of this plane to every box that holds them
-        T* out = a.eb[f];
-        const T* rp = reinterpret_cast<const T*>(sm);
-        const int rs = 2 * pitch;                         // real row stride
-        for (int g = 0; g < d.seg_end - d.seg_begin; ++g) {
-            const Segment& sg = g < kSegSmem ? segs[g] : a.segs[d.seg_begin + g];
-            if (a.own_only && !sg.identity) continue;
-            if (z < sg.z0 || z >= sg.z0 + sg.ez) continue;
-            T* dst = out + sg.dst_off + (int64_t(z + sg.dz) * sg.dLy + sg.y0 + sg.dy) * sg.dLx + sg.x0 + sg.dx;
-            const T* sp = rp + sg.y0 * rs + sg.x0;
-            if (!sg.vec4) {
-                loop2(sg.ex, sg.ey, [&](int yy, int xx) { __stcs(dst + int64_t(yy) * sg.dLx + xx, sp[yy * rs + xx]); });
-            } else if (!store_rows_pow2<kThreads>(dst, sg.dLx, sp, rs, sg.ex >> 2, sg.ey)) {
-                loop2(sg.ex >> 2, sg.ey, [&](int yy, int x4) {
-                    const cpx<T> u = *reinterpret_cast<const cpx<T>*>(sp + yy * rs + 4 * x4);
-                    const cpx<T> w = *reinterpret_cast<const cpx<T>*>(sp + yy * rs + 4 * x4 + 2);
-                    stcs4(dst + int64_t(yy) * sg.dLx + 4 * x4, cpx4<T>{u.x, u.y, w.x, w.y});
-                });
-            }
-        }
+        store_plane<kThreads>(a, d, z, 0, Ly, 0, rs, &plan, kThreads / 32 - 1, a.eb[f], reinterpret_cast<const T*>(sm));
         __syncthreads();
     }
 }
@@ -1036,11 +1098,11 @@ __global__ void __launch_bounds__(kThreads) k_cols(Args<T> a) {
 // stage 7: real merge and inverse x transforms of a block of valid rows of one
 // output plane, then the store of pass C (own box and every guard image)
 template <typename T>
-__global__ void __launch_bounds__(kThreads) k_rows_inv(Args<T> a) {
+__global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? PSATD_MINB_ROWS : 2) k_rows_inv(Args<T> a) {
     extern __shared__ __align__(16) unsigned char smraw[];
     cpx<T>* sm = reinterpret_cast<cpx<T>*>(smraw);
     __shared__ SubDesc d;
-    __shared__ Segment segs[kSegSmem];
+    __shared__ StorePlan plan;
     __shared__ int64_t s_ticket[2];
     Tickets<T> tk(a, s_ticket);
     for (int64_t it = tk.current(); it >= 0; tk.advance(), it = tk.current()) {
@@ -1055,38 +1117,14 @@ __global__ void __launch_bounds__(kThreads) k_rows_inv(Args<T> a) {
         const int h = g.h, pitch = g.pitch, lxh = g.lxh;
         const cpx<T>* src = a.spec + d.spec_off + int64_t(f * g.Lz + z) * g.q + int64_t(ya) * lxh;
         loop2(lxh, nr, [&](int y, int c) { cp_async_c(sm + y * pitch + c, src + y * lxh + c); });
-        const int nsg = min(d.seg_end - d.seg_begin, kSegSmem);
-        {
-            const int* gs = reinterpret_cast<const int*>(a.segs + d.seg_begin);
-            int* ss = reinterpret_cast<int*>(segs);
-            for (int i = threadIdx.x; i < nsg * int(sizeof(Segment) / 4); i += kThreads) ss[i] = __ldg(gs + i);
-        }
+        const int rs = 2 * pitch;                         // real row stride
+        if (threadIdx.x >= kThreads - 32) plan_stores(a, d, d.seg_begin, z, ya, ya + nr, ya, rs, &plan);
         cp_async_wait_all();
         __syncthreads();
         real_merge_rows(sm, nr, pitch, h, g.ax, a.tw + d.tw_post);
         __syncthreads();
         fft_inv<false>(sm, g.ax, Batch{nr, pitch, 0, 0, 1, 1}, a.tw);
-        T* out = a.eb[f];
-        const T* rp = reinterpret_cast<const T*>(sm);
-        const int rs = 2 * pitch;                         // real row stride
-        for (int k = 0; k < d.seg_end - d.seg_begin; ++k) {
-            const Segment& sg = k < kSegSmem ? segs[k] : a.segs[d.seg_begin + k];
-            if (a.own_only && !sg.identity) continue;
-            if (z < sg.z0 || z >= sg.z0 + sg.ez) continue;
-            const int y_lo = max(sg.y0, ya), y_hi = min(sg.y0 + sg.ey, ya + nr);
-            if (y_lo >= y_hi) continue;
-            T* dst = out + sg.dst_off + (int64_t(z + sg.dz) * sg.dLy + y_lo + sg.dy) * sg.dLx + sg.x0 + sg.dx;
-            const T* sp = rp + (y_lo - ya) * rs + sg.x0;
-            if (!sg.vec4) {
-                loop2(sg.ex, y_hi - y_lo, [&](int yy, int xx) { __stcs(dst + int64_t(yy) * sg.dLx + xx, sp[yy * rs + xx]); });
-            } else if (!store_rows_pow2<kThreads>(dst, sg.dLx, sp, rs, sg.ex >> 2, y_hi - y_lo)) {
-                loop2(sg.ex >> 2, y_hi - y_lo, [&](int yy, int x4) {
-                    const cpx<T> u = *reinterpret_cast<const cpx<T>*>(sp + yy * rs + 4 * x4);
-                    const cpx<T> w = *reinterpret_cast<const cpx<T>*>(sp + yy * rs + 4 * x4 + 2);
-                    stcs4(dst + int64_t(yy) * sg.dLx + 4 * x4, cpx4<T>{u.x, u.y, w.x, w.y});
-                });
-            }
-        }
+        store_plane<kThreads>(a, d, z, ya, ya + nr, ya, rs, &plan, kThreads / 32 - 1, a.eb[f], reinterpret_cast<const T*>(sm));
         __syncthreads();
     }
 }

@@ -507,7 +507,7 @@ __global__ void __launch_bounds__(kRegThreads, PSATD_MINB_REG) k_pass_c_reg(Args
     extern __shared__ __align__(16) unsigned char smraw[];
     cpx<float>* sm = reinterpret_cast<cpx<float>*>(smraw);
     __shared__ SubDesc d;
-    __shared__ Segment segs[kSegSmem];
+    __shared__ StorePlan plan;
     __shared__ int64_t s_ticket[2];
     __shared__ __align__(8) uint64_t bar;
     __shared__ int s_ok;
@@ -529,12 +529,9 @@ __global__ void __launch_bounds__(kRegThreads, PSATD_MINB_REG) k_pass_c_reg(Args
             mbar_arrive_expect(&bar, bytes);
             bulk_g2s(sm, a.spec + d.spec_off + int64_t(f * Lz + z) * d.q, bytes, &bar);
         }
-        const int nsg = min(d.seg_end - d.seg_begin, kSegSmem);
-        {
-            const int* gs = reinterpret_cast<const int*>(a.segs + d.seg_begin);
-            int* ss = reinterpret_cast<int*>(segs);
-            for (int i = threadIdx.x; i < nsg * int(sizeof(Segment) / 4); i += kRegThreads) ss[i] = __ldg(gs + i);
-        }
+        // where this plane's cells go, found while the copy is under way
+        const int rs = 2 * P;                             // real row stride
+        if (threadIdx.x >= kRegThreads - 32) plan_stores(a, d, d.seg_begin, z, 0, Ly, 0, rs, &plan);
         if (!wait_bulk(&bar, parity, a.err, &s_ok)) return;
         parity ^= 1u;
         // columns c2 and c2 + np (np = ceil(lxh/2)): consecutive lanes touch
@@ -552,25 +549,8 @@ __global__ void __launch_bounds__(kRegThreads, PSATD_MINB_REG) k_pass_c_reg(Args
         }
         __syncthreads();
         // store the valid cells of this plane to every box that holds them
-        float* out = a.eb[f];
-        const float* rp = reinterpret_cast<const float*>(sm);
-        const int rs = 2 * P;                             // real row stride
-        for (int g = 0; g < d.seg_end - d.seg_begin; ++g) {
-            const Segment& sg = g < kSegSmem ? segs[g] : a.segs[d.seg_begin + g];
-            if (a.own_only && !sg.identity) continue;
-            if (z < sg.z0 || z >= sg.z0 + sg.ez) continue;
-            float* dst = out + sg.dst_off + (int64_t(z + sg.dz) * sg.dLy + sg.y0 + sg.dy) * sg.dLx + sg.x0 + sg.dx;
-            const float* sp = rp + sg.y0 * rs + sg.x0;
-            if (!sg.vec4) {
-                loop2n<kRegThreads>(sg.ex, sg.ey, [&](int yy, int xx) { __stcs(dst + int64_t(yy) * sg.dLx + xx, sp[yy * rs + xx]); });
-            } else if (!store_rows_pow2<kRegThreads>(dst, sg.dLx, sp, rs, sg.ex >> 2, sg.ey)) {
-                loop2n<kRegThreads>(sg.ex >> 2, sg.ey, [&](int yy, int x4) {
-                    const cpx<float> u = *reinterpret_cast<const cpx<float>*>(sp + yy * rs + 4 * x4);
-                    const cpx<float> w = *reinterpret_cast<const cpx<float>*>(sp + yy * rs + 4 * x4 + 2);
-                    stcs4(dst + int64_t(yy) * sg.dLx + 4 * x4, cpx4<float>{u.x, u.y, w.x, w.y});
-                });
-            }
-        }
+        store_plane<kRegThreads>(a, d, z, 0, Ly, 0, rs, &plan, kRegThreads / 32 - 1, a.eb[f],
+                                 reinterpret_cast<const float*>(sm));
         __syncthreads();
     }
 }
