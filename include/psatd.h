@@ -97,15 +97,13 @@ extern "C" {
                                      batched kernels even where the ones with
                                      thread-private transforms of compile-time
                                      length apply (see psatd_plane_engine)     */
-#define PSATD_PACKED_Z       0x800 /* FP32: the z/Eq. 1 stage with one thread per
-                                     mode pair and quarter of its z DFTs, the
-                                     two modes of a pair on packed FP32x2
-                                     lanes, for the local z lengths compiled in
-                                     (see psatd_plane_engine).  It executes
-                                     fewer instructions than the default
-                                     batched z/Eq. 1 kernel but holds fewer
-                                     warps per SM, which on 96^3 boxes makes
-                                     it slower; opt-in                        */
+#define PSATD_PACKED_Z       0x800 /* FP32: the z/Eq. 1 stage that holds four z
+                                     positions of a mode and all its fields in
+                                     registers, wherever the local z lengths
+                                     are compiled in (see psatd_plane_engine).
+                                     Without the flag it runs where it is the
+                                     faster one: the heat equation, and
+                                     unstaggered boxes of one z length       */
 #define PSATD_SPLIT_PLANES   0x80 /* split-plane schedule: the x and y transforms
                                      of the forward and inverse plane stages run
                                      as separate row and column launches (five
@@ -326,10 +324,9 @@ int psatd_geometry_variant(psatd_plan_t plan, int32_t* variant);
  * row and a thread a column pair, with the DFT bodies unrolled for the local
  * lengths compiled in (x: 32, 40, 48, 56, 64, 72, 88, 96, 104; y: 32, 48, 64,
  * 80, 96; default factorisations; not with the split-plane schedule);
- * 2 -- the z/Eq. 1 stage is the packed FP32 kernel (PSATD_PACKED_Z) for
- * the local z lengths compiled in (32, 48, 64, 80, 96; default
- * factorisation; an even number of modes per plane; 6 modes per work item;
- * not for PSATD_HEAT).
+ * 2 -- PSATD_PACKED_Z is given and honoured: the local z lengths are compiled
+ * in (32, 48, 64, 80, 96; default factorisation; chunk_b 0 or 6), every plane
+ * has an even number of modes, FP32, not PSATD_HEAT.
  * 0 -- the generic batched kernels throughout.  PSATD_GENERIC_PLANES turns
  * both off. */
 int psatd_plane_engine(psatd_plan_t plan, int32_t* engine);

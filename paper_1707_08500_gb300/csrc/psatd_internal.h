@@ -43,10 +43,10 @@ constexpr int kRegThreads = 128;
 constexpr int kRegX2[] = {32, 40, 48, 56, 64, 72, 88, 96, 104};
 constexpr int kRegY[] = {32, 48, 64, 80, 96};
 constexpr int reg_pitch(int lxh) { return lxh + ((2 - lxh % 4) + 4) % 4; }
-// modes per item of the compiled-length z/Eq. 1 stage (pass B): three pairs,
-// so that the ten fields' pairs fill 30 lanes of a warp; the z lengths it is
-// compiled for are those of kRegY
-constexpr int kRegM = 6;
+// FP32 z stage of psatd_zpass.cuh (for the z lengths in kRegY): modes per work
+// item, and of the heat equation's one or two fields.
+constexpr int kZModes = 8, kZModesHeat = 16;
+constexpr int64_t kZMaxElems = int64_t(1) << 31;   // of a box's coefficient tables and of its spectra (32-bit offsets)
 
 // Cubic local boxes (side L, ng guards, pass-B chunk M, default splits) that
 // have kernels compiled with their geometry fixed at compile time.

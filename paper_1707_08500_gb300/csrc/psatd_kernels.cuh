@@ -67,18 +67,15 @@ struct alignas(4 * sizeof(T)) twd { cpx<T> hi, lo; };
 // FP32 steps against the FP64 oracle: 5.1e-6, and 3.8e-6 with hi + lo
 // products, at twice their cost.
 template <typename T>
-__device__ __forceinline__ twd<T> ld_tw(const twd<T>* p) {
+__device__ __forceinline__ cpx<T> ld_tw(const twd<T>* p) {
     using V = typename vec2<T>::type;
     const V v = __ldg(reinterpret_cast<const V*>(p));
-    twd<T> t;
-    t.hi = mk(v.x, v.y);
-    t.lo = mk(T(0), T(0));
-    return t;
+    return mk(v.x, v.y);
 }
 template <typename T>   // v * w
-__device__ __forceinline__ cpx<T> mul_tw(cpx<T> v, const twd<T>& w) { return cmul(v, w.hi); }
+__device__ __forceinline__ cpx<T> mul_tw(cpx<T> v, cpx<T> w) { return cmul(v, w); }
 template <typename T>   // v * conj(w)
-__device__ __forceinline__ cpx<T> mul_tw_conj(cpx<T> v, const twd<T>& w) { return cmulc(v, w.hi); }
+__device__ __forceinline__ cpx<T> mul_tw_conj(cpx<T> v, cpx<T> w) { return cmulc(v, w); }
 
 template <typename T>
 struct Args {
@@ -254,7 +251,7 @@ __device__ __forceinline__ void dft_runtime(cpx<T>* v, int R, const twd<T>* __re
         for (int r = 1; r < R; ++r) {
             e += k;
             if (e >= R) e -= R;                   // e = r k mod R
-            const twd<T> w = ld_tw(tw_n + e * nR);
+            const cpx<T> w = ld_tw(tw_n + e * nR);
             acc = acc + (INV ? mul_tw_conj(v[r], w) : mul_tw(v[r], w));
         }
         out[k] = acc;
@@ -278,7 +275,7 @@ __device__ __forceinline__ void stage_mid(cpx<T>* sm, const Batch& bt, const Axi
         for (int r = 0; r < f2; ++r) v[r] = p[r * es];
         dft_runtime<INV>(v, f2, tw_n, ax.n / f2);
         for (int r = 0; r < f2; ++r) {
-            const twd<T> w = ld_tw(tw_n + (INV ? (j2 + f3 * r) * k1 : j2 * r * f1));
+            const cpx<T> w = ld_tw(tw_n + (INV ? (j2 + f3 * r) * k1 : j2 * r * f1));
             p[r * es] = INV ? mul_tw_conj(v[r], w) : mul_tw(v[r], w);
         }
     });
@@ -494,10 +491,8 @@ __device__ __forceinline__ const T* field_in(const Args<T>& a, int f) {
 // Every loop body ends with __syncthreads(), which orders the slot writes and
 // reads.
 template <typename T>
-struct Tickets {
+struct TicketDraw {
     const Args<T>& a;
-    int64_t* slot;
-    int par = 0;
     __device__ int64_t draw() const {
         const int64_t k = int64_t(atomicAdd(a.work, 1ull));
         if (k == a.nitems + int64_t(gridDim.x) - 1) *a.work = 0ull;   // the last ticket of the launch
@@ -507,7 +502,19 @@ struct Tickets {
         if (k >= a.nitems + int64_t(gridDim.x)) atomicOr(a.err, 2u);
         return k;
     }
-    __device__ Tickets(const Args<T>& args, int64_t* s) : a(args), slot(s) {
+    // item number of this CTA's first and following tickets, -1 past the last
+    // item (no further ticket may be drawn then)
+    __device__ int64_t item(int64_t k) const { return k < a.nitems ? a.item0 + k : -1; }
+    __device__ int64_t first() const { return item(a.persistent ? draw() : int64_t(blockIdx.x)); }
+    __device__ int64_t next() const { return a.persistent ? item(draw()) : -1; }
+};
+template <typename T>
+struct Tickets : TicketDraw<T> {
+    using TicketDraw<T>::a;
+    using TicketDraw<T>::draw;
+    int64_t* slot;
+    int par = 0;
+    __device__ Tickets(const Args<T>& args, int64_t* s) : TicketDraw<T>{args}, slot(s) {
         if (threadIdx.x == 0) slot[0] = a.persistent ? draw() : int64_t(blockIdx.x);
         __syncthreads();
     }

@@ -22,6 +22,7 @@ cudaError_t launch_stage_f32(int stage, const LaunchCommon& c, int64_t i0, int64
 cudaError_t launch_stage_f64(int stage, const LaunchCommon& c, int64_t i0, int64_t n, int smem, cudaStream_t s);
 cudaError_t launch_gauss_reduce(const void* subs, int nsub, const double* part, double* out, cudaStream_t st);
 cudaError_t launch_stage_reg(int stage, const LaunchCommon& c, int64_t i0, int64_t n, int smem, cudaStream_t s);
+cudaError_t launch_stage_z(int zlen, bool heat, bool stag, const LaunchCommon& c, int64_t i0, int64_t n, int smem, cudaStream_t s);
 }  // namespace psatd
 
 using namespace psatd;
@@ -202,7 +203,9 @@ struct psatd_plan_s {
     int smemA = 0, smemB = 0, smemC = 0, smemR = 0, smemK = 0;
     bool split = false;                // split-plane schedule (row and column launches)
     bool reg = false;                  // FP32 plane stages with compile-time-length transforms
-    bool regB = false;                 // FP32 z/Eq. 1 stage with compile-time-length transforms
+    bool regB = false;                 // PSATD_PACKED_Z honoured (reported by psatd_plane_engine)
+    bool zpass = false;                // FP32 z stage of psatd_zpass.cuh (else the generic one)
+    int zlen = 0;                      // its z length when every box has the same, else 0
     int smemAreg = 0, smemCreg = 0;
     // workspace layout (bytes)
     size_t off_desc = 0, off_seg = 0, off_tw = 0, off_tab = 0, off_tabc = 0, off_gauss = 0, off_work = 0, off_spec = 0, ws_need = 0;
@@ -549,28 +552,38 @@ int psatd_plan_create_tuned(psatd_plan_t* out, const int32_t global_n[3], const 
     }
     // --- pass-B chunk, shared memory, work items --------------------------------
     const int csz = p->f64 ? 16 : 8;
-    // FP32 z/Eq. 1 stage with compile-time-length z transforms: every local z
-    // length compiled in, the default z factorisation, an even number of
-    // modes per plane, kRegM modes per item
-    if ((flags & PSATD_PACKED_Z) && !p->f64 && !p->heat && !(flags & PSATD_GENERIC_PLANES) &&
-        (!tuning || !tuning->chunk_b || tuning->chunk_b == kRegM)) {
-        bool ok = true;
+    // FP32: the z stage of psatd_zpass.cuh for z lengths in kRegY at their
+    // default split (offsets inside a box in 32 bits) and the default chunk, or
+    // that same one asked for: for the heat equation, and for Maxwell plans
+    // whose boxes share one z length and that are not staggered -- with mixed
+    // lengths it takes 528 us against the generic stage's 512 on uneven48.
+    if (!p->f64 && !(flags & PSATD_GENERIC_PLANES)) {
+        bool set = true, same = true, even = true;
+        const SubDesc& d0 = p->desc[0];
         for (const SubDesc& d : p->desc) {
             bool in = false;
             for (int v : kRegY) in = in || v == d.L[2];
-            ok = ok && in && d.az.f1 == split_first(d.L[2]) && d.q % 2 == 0;   // 16-byte mode pairs
+            set = set && in && d.az.f1 == split_first(d.L[2]) && std::max(p->nf, int(TAB_N)) * int64_t(d.L[2]) * d.q < kZMaxElems;
+            same = same && d.L[2] == d0.L[2];
+            even = even && d.q % 2 == 0;
         }
-        p->regB = ok;
+        const int asked = tuning ? tuning->chunk_b : 0;
+        // PSATD_PACKED_Z asks for it with mixed lengths and staggered fields too
+        // (honoured for an even number of modes per plane)
+        p->regB = (flags & PSATD_PACKED_Z) && set && even && !p->heat && (!asked || asked == 6);
+        p->zpass = p->regB || (set && (p->heat || (same && !p->stag)) && (!asked || asked == (p->heat ? kZModesHeat : kZModes)));
+        p->zlen = same ? d0.L[2] : 0;
     }
     int64_t iA = 0, iB = 0, iC = 0, iA2 = 0, iC1 = 0, spec = 0, maxspec = 0;
     for (int s = 0; s < nsub; ++s) {
         SubDesc& d = p->desc[s];
-        int M = p->regB ? kRegM : (tuning && tuning->chunk_b) ? tuning->chunk_b : (p->f64 ? 4 : 8);
-        if (!p->regB && !(tuning && tuning->chunk_b) && d.L[2] < 16)   // short z pencils (2D): widen up to 512 modes
+        int M = (tuning && tuning->chunk_b) ? tuning->chunk_b : (p->f64 ? 4 : 8);
+        if (!(tuning && tuning->chunk_b) && d.L[2] < 16)   // short z pencils (2D): widen up to 512 modes
             while (M < 512 && int64_t(p->nf) * d.L[2] * (2 * M) * csz <= 48 * 1024) M *= 2;
-        if (!p->regB && !(tuning && tuning->chunk_b) && p->heat)       // one or two fields: wider chunks
+        if (!(tuning && tuning->chunk_b) && p->heat)       // one or two fields: wider chunks
             while (M < 64 && int64_t(p->nf) * d.L[2] * (2 * M) * csz <= 32 * 1024) M *= 2;
-        while (!p->regB && M > 1 && int64_t(p->nf) * (d.L[2] * M + 16) * csz > 200 * 1024) M /= 2;
+        while (M > 1 && int64_t(p->nf) * (d.L[2] * M + 16) * csz > 200 * 1024) M /= 2;
+        if (p->zpass) M = p->heat ? kZModesHeat : kZModes;
         d.chunkB = M;
         d.lgB = 0;
         while ((1 << d.lgB) < M) ++d.lgB;
@@ -587,6 +600,14 @@ int psatd_plan_create_tuned(psatd_plan_t* out, const int32_t global_n[3], const 
         d.spec_off = p->plain ? 0 : spec;
         spec += int64_t(align_up(sp, 32));
         maxspec = std::max<int64_t>(maxspec, int64_t(align_up(sp, 32)));
+    }
+    // the z stage of psatd_zpass.cuh holds E and B twice, every box at the same
+    // field stride
+    if (p->zpass) {
+        int fs = 0;
+        for (const SubDesc& d : p->desc) fs = std::max(fs, d.fsB);
+        for (SubDesc& d : p->desc) d.fsB = fs;
+        p->smemB = (p->nf + p->nout) * fs * csz;
     }
     // planes that do not fit in shared memory take the split-plane schedule:
     // x rows and y columns in separate launches (stages 4-7 of the kernels)
@@ -647,7 +668,7 @@ int psatd_plan_create_tuned(psatd_plan_t* out, const int32_t global_n[3], const 
     if (p->variant < 0 && !p->split) {
         bool dflt = true;
         for (const SubDesc& d : p->desc)
-            dflt = dflt && d.chunkB == (p->f64 ? 4 : 8) && d.ax.f3 <= 1 && d.ay.f3 <= 1 && d.az.f3 <= 1;
+            dflt = dflt && (d.chunkB == (p->f64 ? 4 : 8) || (p->zpass && !p->heat)) && d.ax.f3 <= 1 && d.ay.f3 <= 1 && d.az.f3 <= 1;
         if (dflt) p->variant = -2;
     }
     if (p->smemB > kPlaneSmemMax || (p->split && std::max(p->smemR, p->smemK) > kPlaneSmemMax))
@@ -1041,8 +1062,9 @@ static int launch_push(psatd_plan_s* p, LaunchCommon c, double* gauss_dev, cudaS
             if ((e = stage(p, 5, c, r.a20, r.a2n, p->smemK, s)) != cudaSuccess) return cuda_fail(p, e, "y columns launch");
         }
         if (!p->plain && (e = mark(1)) != cudaSuccess) return cuda_fail(p, e, "event record");
-        if (p->regB) {
-            if ((e = launch_stage_reg(1, c, r.b0, r.bn, p->smemB, s)) != cudaSuccess) return cuda_fail(p, e, "pass B launch");
+        if (p->zpass) {
+            if ((e = launch_stage_z(p->zlen, p->heat, p->stag, c, r.b0, r.bn, p->smemB, s)) != cudaSuccess)
+                return cuda_fail(p, e, "pass B launch");
         } else if ((e = stage(p, p->heat ? 8 : 1, c, r.b0, r.bn, p->smemB, s)) != cudaSuccess) {
             return cuda_fail(p, e, "pass B launch");
         }

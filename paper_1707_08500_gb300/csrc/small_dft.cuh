@@ -325,6 +325,8 @@ template <bool INV> struct Dft<12, INV> : DftSplit<12, 4, INV> {};
 template <bool INV> struct Dft<14, INV> : DftSplit<14, 2, INV> {};
 template <bool INV> struct Dft<15, INV> : DftSplit<15, 3, INV> {};
 template <bool INV> struct Dft<16, INV> : DftSplit<16, 4, INV> {};
+template <bool INV> struct Dft<20, INV> : DftSplit<20, 4, INV> {};
+template <bool INV> struct Dft<24, INV> : DftSplit<24, 3, INV> {};
 
 // Call f(integral_constant<int, n>) for a runtime n in 1..16.
 template <class F>

@@ -1,0 +1,85 @@
+"""The FP32 z stage with a mode's block of four positions in registers
+(psatd_zpass.cuh) against the FP64 oracle: every compiled z length, planes with
+an odd number of modes and a ragged last chunk, the Gauss sums; staggered fields
+and mixed lengths (PSATD_PACKED_Z); the heat equation.  Tolerances: one FP32
+step, 2e-6 relative L2 (measured 2.5e-7); Gauss sums 1e-3 (cancellation in
+i[k].E - rho)."""
+import dataclasses
+
+import numpy as np
+import pytest
+import torch
+
+from oracle import heat_oracle as H
+from oracle import psatd_oracle as O
+from paper_1707_08500_gb300 import inputs as I
+
+pytestmark = pytest.mark.gpu
+NG = 4
+
+
+@pytest.fixture(scope="module")
+def P():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1707_08500_gb300 import build
+    build.build()
+    from paper_1707_08500_gb300 import psatd
+    return psatd
+
+
+def _wl(ycuts, zlens, staggered=False):
+    zc = tuple(v - 2 * NG for v in zlens)
+    wl = I.custom("z", (14, sum(ycuts), sum(zc)), ((14,), ycuts, zc), NG, 8, fields="wavepacket", c_dt=0.6,
+                  precision="f32")
+    return dataclasses.replace(wl, staggered=staggered)
+
+
+def _step(P, wl, flags=0):
+    glob = I.global_fields(wl)
+    sol = P.Solver(wl, gauss=True, extra_flags=flags)
+    sol.load_global(glob, guards=True)
+    sol.push()
+    torch.cuda.synchronize()
+    assert P.psatd_check(sol.plan) == 0
+    gs = []
+    ref = O.step({k: v.numpy() for k, v in glob.items()}, wl, gauss_out=gs)
+    assert O.rel_l2({k: v.numpy() for k, v in sol.gather_global().items()}, ref) < 2e-6
+    np.testing.assert_allclose(sol.gauss_sums(), np.array(gs), rtol=1e-3)
+
+
+# local x 22 (12 columns), y 15: 180 modes per plane, 4 in the last chunk of 8
+@pytest.mark.parametrize("lz", [32, 48, 64, 80, 96])
+@pytest.mark.parametrize("ycuts", [(7,), (8, 5)])
+def test_z_lengths(P, lz, ycuts):
+    _step(P, _wl(ycuts, (lz,)))
+
+
+@pytest.mark.parametrize("lz", [32, 96])
+def test_odd_modes_per_plane(P, lz):
+    # local x 20 (11 columns), y 13: 143 modes
+    wl = I.custom("zodd", (12, 5, lz - 2 * NG), ((12,), (5,), (lz - 2 * NG,)), NG, 8, fields="wavepacket", precision="f32")
+    assert wl.subs[0].local[1] * (wl.subs[0].local[0] // 2 + 1) % 2 == 1
+    _step(P, wl)
+
+
+@pytest.mark.parametrize("zlens,staggered", [((32, 80), False), ((48,), True), ((64, 96), True)])
+def test_mixed_lengths_and_stagger(P, zlens, staggered):
+    wl = _wl((8,), zlens, staggered)
+    assert P.psatd_plane_engine(P.Solver(wl, extra_flags=P.PSATD_PACKED_Z).plan) & 2
+    _step(P, wl, P.PSATD_PACKED_Z)
+
+
+@pytest.mark.parametrize("zlens", [(32,), (48, 64), (80, 96)])
+@pytest.mark.parametrize("source", [False, True])
+@pytest.mark.parametrize("ycuts", [(5,), (8, 7)])
+def test_heat(P, zlens, source, ycuts):
+    wl = _wl(ycuts, zlens)
+    g = I.random_fields(wl.global_n, 3, names=("Jx", "Jy"))
+    names = ("T", "S") if source else ("T",)
+    hs = P.HeatSolver(wl, 0.4, source=source)
+    hs.load_global({"T": g["Jx"], "S": g["Jy"]}, names=names, guards=True)
+    hs.push()
+    torch.cuda.synchronize()
+    ref = H.heat_step({"T": g["Jx"].numpy(), **({"S": g["Jy"].numpy()} if source else {})}, wl, 0.4)["T"]
+    assert H.rel_l2(hs.gather_global(names=("T",))["T"].numpy(), ref) < 2e-6
