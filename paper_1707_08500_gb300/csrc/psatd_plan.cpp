@@ -23,6 +23,7 @@ cudaError_t launch_stage_f64(int stage, const LaunchCommon& c, int64_t i0, int64
 cudaError_t launch_gauss_reduce(const void* subs, int nsub, const double* part, double* out, cudaStream_t st);
 cudaError_t launch_stage_reg(int stage, const LaunchCommon& c, int64_t i0, int64_t n, int smem, cudaStream_t s);
 cudaError_t launch_stage_z(int zlen, bool heat, bool stag, const LaunchCommon& c, int64_t i0, int64_t n, int smem, cudaStream_t s);
+cudaError_t launch_stage_flat(bool stag, const LaunchCommon& c, int64_t i0, int64_t n, cudaStream_t s);
 }  // namespace psatd
 
 using namespace psatd;
@@ -205,6 +206,7 @@ struct psatd_plan_s {
     bool reg = false;                  // FP32 plane stages with compile-time-length transforms
     bool regB = false;                 // PSATD_PACKED_Z honoured (reported by psatd_plane_engine)
     bool zpass = false;                // FP32 z stage of psatd_zpass.cuh (else the generic one)
+    bool flat = false;                 // FP32, every box one cell deep: Eq. 1 without a z transform
     int zlen = 0;                      // its z length when every box has the same, else 0
     int smemAreg = 0, smemCreg = 0;
     // workspace layout (bytes)
@@ -573,6 +575,9 @@ int psatd_plan_create_tuned(psatd_plan_t* out, const int32_t global_n[3], const 
         p->regB = (flags & PSATD_PACKED_Z) && set && even && !p->heat && (!asked || asked == 6);
         p->zpass = p->regB || (set && (p->heat || (same && !p->stag)) && (!asked || asked == (p->heat ? kZModesHeat : kZModes)));
         p->zlen = same ? d0.L[2] : 0;
+        // boxes one cell deep (2D problems) take Eq. 1 alone, for any chunk
+        p->flat = !p->heat;
+        for (const SubDesc& d : p->desc) p->flat = p->flat && d.L[2] == 1 && TAB_N * int64_t(d.q) < kZMaxElems;
     }
     int64_t iA = 0, iB = 0, iC = 0, iA2 = 0, iC1 = 0, spec = 0, maxspec = 0;
     for (int s = 0; s < nsub; ++s) {
@@ -1065,6 +1070,8 @@ static int launch_push(psatd_plan_s* p, LaunchCommon c, double* gauss_dev, cudaS
         if (p->zpass) {
             if ((e = launch_stage_z(p->zlen, p->heat, p->stag, c, r.b0, r.bn, p->smemB, s)) != cudaSuccess)
                 return cuda_fail(p, e, "pass B launch");
+        } else if (p->flat) {
+            if ((e = launch_stage_flat(p->stag, c, r.b0, r.bn, s)) != cudaSuccess) return cuda_fail(p, e, "pass B launch");
         } else if ((e = stage(p, p->heat ? 8 : 1, c, r.b0, r.bn, p->smemB, s)) != cudaSuccess) {
             return cuda_fail(p, e, "pass B launch");
         }

@@ -3,6 +3,13 @@
 
 namespace psatd {
 
+// Eq. 1 of boxes one cell deep along z.
+cudaError_t launch_stage_flat(bool stag, const LaunchCommon& c, int64_t item0, int64_t nitems, cudaStream_t st) {
+    if (nitems <= 0) return cudaSuccess;
+    const Args<float> a = make_args<float>(c, item0, nitems);
+    return stag ? launch_kernel<float>(k_pass_b_flat<true>, a, 0, st) : launch_kernel<float>(k_pass_b_flat<false>, a, 0, st);
+}
+
 cudaError_t launch_stage_z(int zlen, bool heat, bool stag, const LaunchCommon& c, int64_t item0, int64_t nitems, int smem,
                            cudaStream_t st) {
     if (nitems <= 0) return cudaSuccess;

@@ -83,3 +83,13 @@ def test_heat(P, zlens, source, ycuts):
     torch.cuda.synchronize()
     ref = H.heat_step({"T": g["Jx"].numpy(), **({"S": g["Jy"].numpy()} if source else {})}, wl, 0.4)["T"]
     assert H.rel_l2(hs.gather_global(names=("T",))["T"].numpy(), ref) < 2e-6
+
+
+@pytest.mark.parametrize("staggered", [False, True])
+@pytest.mark.parametrize("cuts", [((14,), (5,)), ((24, 56), (16, 34, 7))])
+def test_one_cell_deep(P, staggered, cuts):
+    # 2D problems: Eq. 1 without a z transform; 143 modes in one chunk, then
+    # several chunks of 512 and ragged ones
+    wl = I.custom("flat", (sum(cuts[0]), sum(cuts[1]), 1), cuts + ((1,),), NG, 8, fields="wavepacket", precision="f32",
+                  two_d=True)
+    _step(P, dataclasses.replace(wl, staggered=staggered))
