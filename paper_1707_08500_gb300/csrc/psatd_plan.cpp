@@ -21,7 +21,7 @@ namespace psatd {
 cudaError_t launch_stage_f32(int stage, const LaunchCommon& c, int64_t i0, int64_t n, int smem, cudaStream_t s);
 cudaError_t launch_stage_f64(int stage, const LaunchCommon& c, int64_t i0, int64_t n, int smem, cudaStream_t s);
 cudaError_t launch_gauss_reduce(const void* subs, int nsub, const double* part, double* out, cudaStream_t st);
-cudaError_t launch_stage_reg(int stage, const LaunchCommon& c, int64_t i0, int64_t n, int smem, cudaStream_t s);
+cudaError_t launch_stage_reg(int stage, int rows, const LaunchCommon& c, int64_t i0, int64_t n, int smem, cudaStream_t s);
 cudaError_t launch_stage_z(int zlen, bool heat, bool stag, const LaunchCommon& c, int64_t i0, int64_t n, int smem, cudaStream_t s);
 cudaError_t launch_stage_flat(bool stag, const LaunchCommon& c, int64_t i0, int64_t n, cudaStream_t s);
 }  // namespace psatd
@@ -208,7 +208,7 @@ struct psatd_plan_s {
     bool zpass = false;                // FP32 z stage of psatd_zpass.cuh (else the generic one)
     bool flat = false;                 // FP32, every box one cell deep: Eq. 1 without a z transform
     int zlen = 0;                      // its z length when every box has the same, else 0
-    int smemAreg = 0, smemCreg = 0;
+    int smemAreg = 0, smemCreg = 0, regRows = 0;
     // workspace layout (bytes)
     size_t off_desc = 0, off_seg = 0, off_tw = 0, off_tab = 0, off_tabc = 0, off_gauss = 0, off_work = 0, off_spec = 0, ws_need = 0;
     size_t off_io = 0, off_io_map = 0;
@@ -688,7 +688,8 @@ int psatd_plan_create_tuned(psatd_plan_t* out, const int32_t global_n[3], const 
             ok = ok && listed(kRegX2, int(sizeof(kRegX2) / sizeof(int)), d.L[0]) &&
                  listed(kRegY, int(sizeof(kRegY) / sizeof(int)), d.L[1]) && d.ax.f1 == split_first(d.L[0] / 2) &&
                  d.ay.f1 == split_first(d.L[1]) && d.lxh <= kRegThreads / 2 && d.L[1] <= kRegThreads;
-            p->smemAreg = std::max(p->smemAreg, d.L[1] * reg_pitch(d.lxh) * 8);
+            p->smemAreg = std::max(p->smemAreg, d.L[1] * reg_pitch(d.L[0] / 2) * 8);
+            p->regRows = std::max(p->regRows, d.L[1]);
             p->smemCreg = std::max(p->smemCreg, d.q * 8);
         }
         p->reg = ok && p->smemAreg <= kPlaneSmemMax && p->smemCreg <= kPlaneSmemMax;
@@ -1059,7 +1060,7 @@ static int launch_push(psatd_plan_s* p, LaunchCommon c, double* gauss_dev, cudaS
     struct Range { int64_t a0, an, a20, a2n, b0, bn, c10, c1n, c0, cn; };
     auto run = [&](const Range& r) -> int {
         if (p->reg) {
-            if ((e = launch_stage_reg(0, c, r.a0, r.an, p->smemAreg, s)) != cudaSuccess) return cuda_fail(p, e, "pass A launch");
+            if ((e = launch_stage_reg(0, p->regRows, c, r.a0, r.an, p->smemAreg, s)) != cudaSuccess) return cuda_fail(p, e, "pass A launch");
         } else if (!p->split) {
             if ((e = stage(p, 0, c, r.a0, r.an, p->smemA, s)) != cudaSuccess) return cuda_fail(p, e, "pass A launch");
         } else {
@@ -1077,7 +1078,7 @@ static int launch_push(psatd_plan_s* p, LaunchCommon c, double* gauss_dev, cudaS
         }
         if (!p->plain && (e = mark(2)) != cudaSuccess) return cuda_fail(p, e, "event record");
         if (p->reg) {
-            if ((e = launch_stage_reg(2, c, r.c0, r.cn, p->smemCreg, s)) != cudaSuccess) return cuda_fail(p, e, "pass C launch");
+            if ((e = launch_stage_reg(2, p->regRows, c, r.c0, r.cn, p->smemCreg, s)) != cudaSuccess) return cuda_fail(p, e, "pass C launch");
         } else if (!p->split) {
             if ((e = stage(p, 2, c, r.c0, r.cn, p->smemC, s)) != cudaSuccess) return cuda_fail(p, e, "pass C launch");
         } else {

@@ -12,8 +12,9 @@
 //                 and the real split (forward), or the real merge and the
 //                 inverse (pass C), entirely on its own row, so the x phase
 //                 needs no barrier;
-//   y (columns):  a thread works on a pair of half-spectrum columns; the
-//                 four warps (eight half-warps when there are at most 16
+//   y (columns):  a thread works on a pair of half-spectrum columns.  Forward,
+//                 the (pair, DFT) tasks are spread over all threads; inverse,
+//                 the four warps (eight half-warps when there are at most 16
 //                 pairs) take every fourth (eighth) f1-point and f2-point
 //                 DFT of the column pairs.
 //
@@ -30,6 +31,11 @@
 
 #ifndef PSATD_MINB_REG
 #define PSATD_MINB_REG 5
+#endif
+// Threads per SM that pass A's registers are held to (five blocks of 96: as
+// many planes of 96^2 as shared memory holds).
+#ifndef PSATD_REG_THREADS_SM
+#define PSATD_REG_THREADS_SM 480
 #endif
 
 namespace psatd {
@@ -138,8 +144,8 @@ __device__ __forceinline__ void merge_pair_c(cpx<float> A, cpx<float> B, cpx<flo
 }
 
 // Forward real transform of one row: row[0..H) holds z[m] = x[2m] + i x[2m+1]
-// (16-byte aligned); on return row[0..H] holds the half spectrum X[0..H] in
-// position order.
+// (16-byte aligned); on return row[0..H) holds the half spectrum X[0..H) in
+// position order, the real X[0] and X[H] as the two parts of row[0].
 template <int H>
 __device__ __forceinline__ void row_fwd(cpx<float>* row, const twd<float>* __restrict__ tw,
                                         const twd<float>* __restrict__ wp) {
@@ -177,7 +183,7 @@ __device__ __forceinline__ void row_fwd(cpx<float>* row, const twd<float>* __res
         cpx<float> v[F2], o[F2];
         load_dft(0, v);
         const cpx<float> z0 = v[0];
-        o[0] = mk(z0.x + z0.y, 0.f);
+        o[0] = mk(z0.x + z0.y, z0.x - z0.y);
         // positions P and F2 - P hold frequencies F1 P and H - F1 P
 #pragma unroll
         for (int P = 1; P <= F2 / 2; ++P) {
@@ -188,7 +194,6 @@ __device__ __forceinline__ void row_fwd(cpx<float>* row, const twd<float>* __res
         }
 #pragma unroll
         for (int i = 0; i < F2; i += 2) sts4(row + i, o[i], o[i + 1]);
-        row[H] = mk(z0.x - z0.y, 0.f);
     }
     // position k1 F2 + k2 pairs with (F1 - k1) F2 + F2 - 1 - k2
 #pragma unroll 1
@@ -303,17 +308,12 @@ __device__ __forceinline__ void row_inv(cpx<float>* row, const twd<float>* __res
     }
 }
 
-// ---- y: column pairs, four or eight threads per pair ------------------------
-// Thread (pair c2, group q of nq) works on two columns: 2 c2 and 2 c2 + 1 in
-// passes A and B, c2 and c2 + ceil(lxh/2) in pass C (the second may be past
-// the half spectrum: it is then padding, computed on and never stored, or,
-// with `tail` set, neither read nor written); group q takes every nq-th
-// stage-1 (stride) DFT and every nq-th stage-2 (block) DFT.
+// ---- inverse y: column pairs, four or eight threads per pair --------------------
+// Thread (pair c2, group q of nq) works on columns c2 and c2 + ceil(lxh/2) (the
+// second may be past the half spectrum: with `tail` set it is neither read nor
+// written); group q takes every nq-th stage-1 (block) and stage-2 (stride) DFT.
 // tw = exp(-2 pi i m/L), m = 0..L-1.
 
-// element pair (columns c, c + off2) of row y: one 16-byte access for
-// adjacent columns at an even pitch, two 8-byte accesses otherwise (the second
-// skipped for a tail column)
 // Lanes of the y phase: ceil(lxh/2) column pairs, one per lane, in four
 // groups of 32 lanes (the four warps); with at most 16 pairs in eight groups
 // of 16 (half-warps), so that fewer lanes idle on narrow planes.  Group q
@@ -330,69 +330,20 @@ __device__ __forceinline__ int lane_group(int lxh) {
 struct ColPair {
     cpx<float>* base;   // element (0, c)
     int P;              // row pitch (complex)
-    bool v16, tail;
-    int off2;           // the second column: c + off2 (1 with v16)
+    bool tail;
+    int off2;           // the second column: c + off2
     __device__ __forceinline__ void ld(int y, cpx<float>& a, cpx<float>& b) const {
         cpx<float>* q = base + y * P;
-        if (v16) {
-            const float4 v = lds4(q);
-            a = mk(v.x, v.y);
-            b = mk(v.z, v.w);
-        } else {
-            a = q[0];
-            b = tail ? mk(0.f, 0.f) : q[off2];
-        }
+        a = q[0];
+        b = tail ? mk(0.f, 0.f) : q[off2];
     }
     __device__ __forceinline__ void st(int y, cpx<float> a, cpx<float> b) const {
         cpx<float>* q = base + y * P;
-        if (v16) {
-            sts4(q, a, b);
-        } else {
-            q[0] = a;
-            if (!tail) q[off2] = b;
-        }
+        q[0] = a;
+        if (!tail) q[off2] = b;
     }
 };
 
-// forward, stage 1: F1-point DFTs at stride F2, twiddle w^{j r}, in place
-template <int LY>
-__device__ __forceinline__ void col_fwd1(const ColPair& cp, int q, int nq, const twd<float>* __restrict__ tw) {
-    constexpr int F1 = split_first(LY), F2 = LY / F1;
-#pragma unroll 1
-    for (int j = q; j < F2; j += nq) {
-        cpx<float> a[F1], b[F1];
-#pragma unroll
-        for (int r = 0; r < F1; ++r) cp.ld(j + F2 * r, a[r], b[r]);
-        Dft<F1, false>::run(a);
-        Dft<F1, false>::run(b);
-        cp.st(j, a[0], b[0]);
-#pragma unroll
-        for (int r = 1; r < F1; ++r) {
-            const cpx<float> w = ld_tw(tw + j * r);
-            cp.st(j + F2 * r, mul_tw(a[r], w), mul_tw(b[r], w));
-        }
-    }
-}
-// forward, stage 2: F2-point DFTs on contiguous blocks, written to global
-// (row stride `ld` complex, columns c and c+1 at dst[0], dst[1]) in position order
-template <int LY>
-__device__ __forceinline__ void col_fwd2(const ColPair& cp, int q, int nq, cpx<float>* dst, int ld, bool second) {
-    constexpr int F1 = split_first(LY), F2 = LY / F1;
-#pragma unroll 1
-    for (int k = q; k < F1; k += nq) {
-        cpx<float> a[F2], b[F2];
-#pragma unroll
-        for (int r = 0; r < F2; ++r) cp.ld(k * F2 + r, a[r], b[r]);
-        Dft<F2, false>::run(a);
-        Dft<F2, false>::run(b);
-#pragma unroll
-        for (int r = 0; r < F2; ++r) {
-            cpx<float>* d = dst + (k * F2 + r) * ld;
-            stcs_c(d, a[r]);
-            if (second) stcs_c(d + 1, b[r]);
-        }
-    }
-}
 // inverse, stage 1: F2-point DFTs on contiguous blocks, twiddle conj(w^{r k})
 template <int LY>
 __device__ __forceinline__ void col_inv1(const ColPair& cp, int q, int nq, const twd<float>* __restrict__ tw) {
@@ -442,27 +393,100 @@ __device__ __forceinline__ void loop2n(int count, int nouter, F&& f) {
 }
 
 // ---- pass A ------------------------------------------------------------------
+// The y transforms of a plane whose rows hold Lx/2 half-spectrum columns at
+// pitch P (complex): tasks (column pair, DFT) spread over all NT threads, the
+// pair (c, c + np), np = Lx/4, so that consecutive lanes touch consecutive
+// elements.  Stage 1 in place; stage 2 to global memory (rows of ld complex)
+// in position order, column 0 to c0 instead.
+template <int LY, int NT>
+__device__ __forceinline__ void cols_fwd1(cpx<float>* sm, int P, int np, const twd<float>* __restrict__ tw) {
+    constexpr int F1 = split_first(LY), F2 = LY / F1;
+    loop2n<NT>(np, F2, [&](int j, int c) {
+        cpx<float>* q = sm + j * P + c;
+        const int st = F2 * P;
+        cpx<float> a[F1], b[F1];
+#pragma unroll
+        for (int r = 0; r < F1; ++r) {
+            a[r] = q[r * st];
+            b[r] = q[r * st + np];
+        }
+        Dft<F1, false>::run(a);
+        Dft<F1, false>::run(b);
+        q[0] = a[0];
+        q[np] = b[0];
+#pragma unroll
+        for (int r = 1; r < F1; ++r) {
+            const cpx<float> w = ld_tw(tw + j * r);
+            q[r * st] = mul_tw(a[r], w);
+            q[r * st + np] = mul_tw(b[r], w);
+        }
+    });
+}
+template <int LY, int NT>
+__device__ __forceinline__ void cols_fwd2(const cpx<float>* sm, int P, int np, cpx<float>* dst, int ld, cpx<float>* c0) {
+    constexpr int F1 = split_first(LY), F2 = LY / F1;
+    loop2n<NT>(np, F1, [&](int k, int c) {
+        const cpx<float>* q = sm + k * F2 * P + c;
+        cpx<float> a[F2], b[F2];
+#pragma unroll
+        for (int r = 0; r < F2; ++r) {
+            a[r] = q[r * P];
+            b[r] = q[r * P + np];
+        }
+        Dft<F2, false>::run(a);
+        Dft<F2, false>::run(b);
+        cpx<float>* d = dst + k * F2 * ld + c;
+#pragma unroll
+        for (int r = 0; r < F2; ++r) {
+            if (c) stcs_c(d + r * ld, a[r]);
+            else c0[k * F2 + r] = a[r];
+            stcs_c(d + r * ld + np, b[r]);
+        }
+    });
+}
+
 // Work item (subdomain, field, z plane): the plane's rows are copied to shared
-// memory at pitch reg_pitch(Lx/2+1); thread y transforms row y along x; then
-// two threads per column transform along y and store the half spectrum.
-__global__ void __launch_bounds__(kRegThreads, PSATD_MINB_REG) k_pass_a_reg(Args<float> a) {
+// memory at pitch reg_pitch(Lx/2); thread y transforms row y along x; then the
+// column pairs are transformed along y and the half spectrum stored.  The real
+// columns 0 and Lx/2 go through the y transform as the two parts of one complex
+// column, whose spectrum splits by conjugate symmetry, so that Lx/2 columns and
+// not Lx/2 + 1 share out evenly: on 96^2 planes three warps have one row and
+// then two and three DFT pairs per thread.  That split is done while the next
+// plane arrives.  Bound: issue (54% of cycles, 15 warps per SM) and HBM (54%).
+// 512 boxes of 96^3, ten fields: 8.76 ms with four warps, a lane per column
+// pair and 49 columns, 8.21 ms so; on mixed boxes the same within 1%.  Bulk
+// prefetches of the planes ahead into L2 gain nothing.
+template <int NT>
+__global__ void __launch_bounds__(NT, PSATD_REG_THREADS_SM / NT) k_pass_a_reg(Args<float> a) {
     extern __shared__ __align__(16) unsigned char smraw[];
     cpx<float>* sm = reinterpret_cast<cpx<float>*>(smraw);
     __shared__ SubDesc d;
     __shared__ int64_t s_ticket[2];
     __shared__ __align__(8) uint64_t bar;
     __shared__ int s_ok;
+    __shared__ cpx<float> c0[NT];              // column 0 of the last plane, position order
     if (threadIdx.x == 0) mbar_init(&bar, 1);
     __syncthreads();
     unsigned parity = 0;
+    cpx<float>* dst0 = nullptr;                // the last plane's spectrum, and its shape
+    int h0 = 0, L0 = 0, f10 = 1, f20 = 1;
+    auto split0 = [&]() {
+        for (int p = int(threadIdx.x); p < L0; p += NT) {
+            const int k1 = p / f20, k2 = p - k1 * f20;          // ky = k1 + f1 k2; -ky:
+            const int pm = k1 ? (f10 - k1) * f20 + f20 - 1 - k2 : k2 ? f20 - k2 : 0;
+            const cpx<float> u = c0[p], v = c0[pm];
+            stcs_c(dst0 + p * (h0 + 1), mk(0.5f * (u.x + v.x), 0.5f * (u.y - v.y)));
+            stcs_c(dst0 + p * (h0 + 1) + h0, mk(0.5f * (u.y + v.y), 0.5f * (v.x - u.x)));
+        }
+    };
     Tickets<float> tk(a, s_ticket);
     for (int64_t it = tk.current(); it >= 0; tk.advance(), it = tk.current()) {
         tk.prefetch();
         decode_item<0>(a, it, &d);
-        const int Lx = d.L[0], Ly = d.L[1], Lz = d.L[2], lxh = d.lxh;
+        const int Lx = d.L[0], Ly = d.L[1], Lz = d.L[2], h = Lx >> 1;
         const int loc = int(it - d.itemA);
         const int f = loc / Lz, z = loc - (loc / Lz) * Lz;
-        const int P = reg_pitch(lxh);
+        const int P = reg_pitch(h);
         const float* src = field_in(a, f) + d.field_off + int64_t(z) * Ly * Lx;
         if (threadIdx.x < 32) {
             if (threadIdx.x == 0) {
@@ -472,6 +496,7 @@ __global__ void __launch_bounds__(kRegThreads, PSATD_MINB_REG) k_pass_a_reg(Args
             __syncwarp();
             for (int y = threadIdx.x; y < Ly; y += 32) bulk_g2s(sm + y * P, src + int64_t(y) * Lx, unsigned(Lx * 4), &bar);
         }
+        split0();
         if (!wait_bulk(&bar, parity, a.err, &s_ok)) return;
         parity ^= 1u;
         if (int(threadIdx.x) < Ly) {
@@ -479,18 +504,15 @@ __global__ void __launch_bounds__(kRegThreads, PSATD_MINB_REG) k_pass_a_reg(Args
             dispatch_x<0>(Lx, [&](auto lc) { row_fwd<decltype(lc)::value / 2>(row, a.tw + d.ax.tw, a.tw + d.tw_post); });
         }
         __syncthreads();
-        // y: lane group q takes every nq-th DFT of column pair (2 c2, 2 c2 + 1)
-        const int c2 = lane_col(lxh), q = lane_group(lxh), nq = lane_groups(lxh);
-        const ColPair cp{sm + 2 * c2, P, true, false, 1};
-        const bool act = 2 * c2 < lxh;
-        if (act) dispatch_y<0>(Ly, [&](auto lc) { col_fwd1<decltype(lc)::value>(cp, q, nq, a.tw + d.ay.tw); });
+        const int np = h >> 1;
+        dispatch_y<0>(Ly, [&](auto lc) { cols_fwd1<decltype(lc)::value, NT>(sm, P, np, a.tw + d.ay.tw); });
         __syncthreads();
-        if (act) {
-            cpx<float>* dst = a.spec + d.spec_off + int64_t(f * Lz + z) * d.q + 2 * c2;
-            dispatch_y<0>(Ly, [&](auto lc) { col_fwd2<decltype(lc)::value>(cp, q, nq, dst, lxh, 2 * c2 + 1 < lxh); });
-        }
+        dst0 = a.spec + d.spec_off + int64_t(f * Lz + z) * d.q;
+        h0 = h; L0 = Ly; f10 = d.ay.f1; f20 = d.ay.f2;
+        dispatch_y<0>(Ly, [&](auto lc) { cols_fwd2<decltype(lc)::value, NT>(sm, P, np, dst0, h + 1, c0); });
         __syncthreads();
     }
+    split0();
 }
 
 // ---- pass C ------------------------------------------------------------------
@@ -534,7 +556,7 @@ __global__ void __launch_bounds__(kRegThreads, PSATD_MINB_REG) k_pass_c_reg(Args
         // columns c2 and c2 + np (np = ceil(lxh/2)): consecutive lanes touch
         // consecutive 8-byte elements, free of bank conflicts at the odd pitch
         const int c2 = lane_col(lxh), q = lane_group(lxh), nq = lane_groups(lxh), np = (lxh + 1) >> 1;
-        const ColPair cp{sm + c2, P, false, c2 + np >= lxh, np};
+        const ColPair cp{sm + c2, P, c2 + np >= lxh, np};
         const bool act = c2 < np;
         if (act) dispatch_y<0>(Ly, [&](auto lc) { col_inv1<decltype(lc)::value>(cp, q, nq, a.tw + d.ay.tw); });
         __syncthreads();
