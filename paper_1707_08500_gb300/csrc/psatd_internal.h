@@ -85,7 +85,7 @@ struct SubDesc {
     int q;               // Ly * lxh: modes per z plane
     AxisPlan ax;         // x: half length h = Lx/2 (complex FFT of packed pairs)
     AxisPlan ay, az;
-    int tw_post;         // offset of exp(-2 pi i k/Lx), k = 0..Lx/2, in the pool
+    int tw_post;         // offset of exp(-2 pi i k/Lx)/2 in position order, in the pool
     int pad0;
     int64_t field_off;   // element offset of the local box in every field arena
     int64_t spec_off;    // complex offset of this subdomain's spectra block

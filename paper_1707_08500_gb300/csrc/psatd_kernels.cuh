@@ -382,6 +382,28 @@ __device__ __forceinline__ void split_pair_ax(int i, int h, const AxisPlan& ax, 
     }
 }
 
+// Real split of one pair of positions of the packed transform: A = Z[pa],
+// B = Z[pb] (pb the partner of pa); X[pa] = e + w o, X[pb] = conj(e - w o) with
+// e = (A + conj B)/2, o = (A - conj B)/(2i), w the real-split twiddle of pa,
+// given halved (wh = w/2): 12 operations, the factor 1/2 of e inside the
+// multiply-adds and that of o in wh, both exact.
+template <typename T>
+__device__ __forceinline__ void split_pair_v(cpx<T> A, cpx<T> B, cpx<T> wh, cpx<T>& outA, cpx<T>& outB) {
+    const cpx<T> s = mk(A.x + B.x, A.y - B.y), d = mk(A.x - B.x, A.y + B.y);
+    const cpx<T> wo = cmul(mk(d.y, -d.x), wh);
+    outA = mk(fma_t(T(0.5), s.x, wo.x), fma_t(T(0.5), s.y, wo.y));
+    outB = mk(fma_t(T(0.5), s.x, -wo.x), fma_t(T(-0.5), s.y, wo.y));
+}
+// Inverse of split_pair_v: X[pa] = A, X[pb] = B -> Z[pa] = e + i o,
+// Z[pb] = conj(e) + i conj(o), e = A + conj B, o = (A - conj B) conj(w).
+template <typename T>
+__device__ __forceinline__ void merge_pair_v(cpx<T> A, cpx<T> B, cpx<T> wh, cpx<T>& outA, cpx<T>& outB) {
+    const cpx<T> e = mk(A.x + B.x, A.y - B.y);
+    const cpx<T> o = cmulc(mk(A.x - B.x, A.y + B.y), wh);
+    outA = mk(fma_t(T(-2), o.y, e.x), fma_t(T(2), o.x, e.y));
+    outB = mk(fma_t(T(2), o.y, e.x), fma_t(T(2), o.x, -e.y));
+}
+
 // Real split after the packed forward x transform: rows r < nrows at
 // p0 + r*pitch hold the h-point transform of z[m] = x[2m] + i x[2m+1] in
 // position order; each becomes the half spectrum X[0..h] of its real row,
@@ -398,13 +420,10 @@ __device__ __forceinline__ void real_split_rows(cpx<T>* p0, int nrows, int pitch
         } else {
             int pa, pb;
             split_pair_ax(i, h, ax, pa, pb);
-            const cpx<T> A = p[pa], Bc = conj(p[pb]);
-            const cpx<T> e = scale(A + Bc, T(0.5));
-            const cpx<T> dd = A - Bc;
-            const cpx<T> o = mk(T(0.5) * dd.y, T(-0.5) * dd.x);   // (A - conj B)/(2i)
-            const cpx<T> wo = mul_tw(o, ld_tw(wp + pa));
-            p[pa] = e + wo;
-            if (pb != pa) p[pb] = conj(e - wo);
+            cpx<T> oa, ob;
+            split_pair_v(p[pa], p[pb], ld_tw(wp + pa), oa, ob);
+            p[pa] = oa;
+            if (pb != pa) p[pb] = ob;
         }
     });
 }
@@ -423,11 +442,10 @@ __device__ __forceinline__ void real_merge_rows(cpx<T>* p0, int nrows, int pitch
         } else {
             int pa, pb;
             split_pair_ax(i, h, ax, pa, pb);
-            const cpx<T> A = p[pa], Bc = conj(p[pb]);
-            const cpx<T> e = A + Bc;
-            const cpx<T> o = mul_tw_conj(A - Bc, ld_tw(wp + pa));
-            p[pa] = e + mul_i(o);
-            if (pb != pa) p[pb] = conj(e) + mul_i(conj(o));
+            cpx<T> oa, ob;
+            merge_pair_v(p[pa], p[pb], ld_tw(wp + pa), oa, ob);
+            p[pa] = oa;
+            if (pb != pa) p[pb] = ob;
         }
     });
 }
@@ -750,47 +768,82 @@ __device__ __forceinline__ void eq1_mode(const Args<T>& a, const SubDesc& d, cpx
     const T omCk = __ldg(tb + 4 * NM), Dk = __ldg(tb + 5 * NM), inv = __ldg(tb + 6 * NM);
     const T kx = __ldg(tk + xp), ky = __ldg(tk + lxh + yp), kz = __ldg(tk + lxh + Ly + zp);
     const T hx = kx * inv, hy = ky * inv, hz = kz * inv;
-    cpx<T> E0 = p[0], E1 = p[fs], E2 = p[2 * fs];
-    cpx<T> B0 = p[3 * fs], B1 = p[4 * fs], B2 = p[5 * fs];
-    cpx<T> J0 = p[6 * fs], J1 = p[7 * fs], J2 = p[8 * fs];
-    cpx<T> px, py, pz;
-    if (a.staggered) {
-        const cpx<T>* ph = a.tabc + d.tab_ph;
-        px = ldg_c(ph + xp); py = ldg_c(ph + lxh + yp); pz = ldg_c(ph + lxh + Ly + zp);
-        const cpx<T> pyz = cmul(py, pz), pxz = cmul(px, pz), pxy = cmul(px, py);
-        E0 = cmul(E0, px); E1 = cmul(E1, py); E2 = cmul(E2, pz);
-        J0 = cmul(J0, px); J1 = cmul(J1, py); J2 = cmul(J2, pz);
-        B0 = cmul(B0, pyz); B1 = cmul(B1, pxz); B2 = cmul(B2, pxy);
-    }
-    // khat x B, khat x E, khat x J, khat.E, khat.J
-    const cpx<T> hB0 = scale(B2, hy) - scale(B1, hz), hB1 = scale(B0, hz) - scale(B2, hx), hB2 = scale(B1, hx) - scale(B0, hy);
-    const cpx<T> hE0 = scale(E2, hy) - scale(E1, hz), hE1 = scale(E0, hz) - scale(E2, hx), hE2 = scale(E1, hx) - scale(E0, hy);
-    const cpx<T> hJ0 = scale(J2, hy) - scale(J1, hz), hJ1 = scale(J0, hz) - scale(J2, hx), hJ2 = scale(J1, hx) - scale(J0, hy);
-    const cpx<T> dE = scale(E0, hx) + scale(E1, hy) + scale(E2, hz);
-    const cpx<T> dJ = scale(J0, hx) + scale(J1, hy) + scale(J2, hz);
-    // Eq. 1a: E' = C E + i S khat x B - S/k J + (1-C) khat (khat.E) + khat (khat.J)(S/k - dt)
-    const cpx<T> lo = scale(dE, omC) + scale(dJ, Dk);
-    cpx<T> F0 = scale(E0, C) + scale(mul_i(hB0), S) - scale(J0, Sk) + scale(lo, hx);
-    cpx<T> F1 = scale(E1, C) + scale(mul_i(hB1), S) - scale(J1, Sk) + scale(lo, hy);
-    cpx<T> F2 = scale(E2, C) + scale(mul_i(hB2), S) - scale(J2, Sk) + scale(lo, hz);
+    const cpx<T> E0 = p[0], E1 = p[fs], E2 = p[2 * fs];
+    const cpx<T> B0 = p[3 * fs], B1 = p[4 * fs], B2 = p[5 * fs];
+    const cpx<T> J0 = p[6 * fs], J1 = p[7 * fs], J2 = p[8 * fs];
+    // Eq. 1a: E' = C E + i S khat x B - S/k J + khat [(1-C) khat.E + (S/k - dt) khat.J]
     // Eq. 1b: B' = C B - i S khat x E + i (1-C)/k khat x J
-    cpx<T> G0 = scale(B0, C) - scale(mul_i(hE0), S) + scale(mul_i(hJ0), omCk);
-    cpx<T> G1 = scale(B1, C) - scale(mul_i(hE1), S) + scale(mul_i(hJ1), omCk);
-    cpx<T> G2 = scale(B2, C) - scale(mul_i(hE2), S) + scale(mul_i(hJ2), omCk);
+    // component a from its cyclic neighbours b, c: (khat x F)_a = h_b F_c - h_c F_b
+    cpx<T> F0, F1, F2, G0, G1, G2;
+    T sx, sy;                      // [k].E' in nodal position
+    if (!a.staggered) {
+        const T Sx = S * hx, Sy = S * hy, Sz = S * hz, Kx = omCk * hx, Ky = omCk * hy, Kz = omCk * hz;
+        auto dot = [&](T u, T v, T w) { return fma_t(u, hx, fma_t(v, hy, w * hz)); };
+        const T lx = fma_t(omC, dot(E0.x, E1.x, E2.x), Dk * dot(J0.x, J1.x, J2.x));
+        const T ly = fma_t(omC, dot(E0.y, E1.y, E2.y), Dk * dot(J0.y, J1.y, J2.y));
+        auto new_e = [&](cpx<T> Ea, cpx<T> Bb, cpx<T> Bc, cpx<T> Ja, T h, T Sb, T Sc) {
+            return mk(fma_t(C, Ea.x, fma_t(-Sb, Bc.y, fma_t(Sc, Bb.y, fma_t(-Sk, Ja.x, h * lx)))),
+                      fma_t(C, Ea.y, fma_t(Sb, Bc.x, fma_t(-Sc, Bb.x, fma_t(-Sk, Ja.y, h * ly)))));
+        };
+        auto new_b = [&](cpx<T> Ba, cpx<T> Eb, cpx<T> Ec, cpx<T> Jb, cpx<T> Jc, T Sb, T Sc, T Kb, T Kc) {
+            return mk(fma_t(C, Ba.x, fma_t(Sb, Ec.y, fma_t(-Sc, Eb.y, fma_t(-Kb, Jc.y, Kc * Jb.y)))),
+                      fma_t(C, Ba.y, fma_t(-Sb, Ec.x, fma_t(Sc, Eb.x, fma_t(Kb, Jc.x, -Kc * Jb.x)))));
+        };
+        F0 = new_e(E0, B1, B2, J0, hx, Sy, Sz);
+        F1 = new_e(E1, B2, B0, J1, hy, Sz, Sx);
+        F2 = new_e(E2, B0, B1, J2, hz, Sx, Sy);
+        G0 = new_b(B0, E1, E2, J1, J2, Sy, Sz, Ky, Kz);
+        G1 = new_b(B1, E2, E0, J2, J0, Sz, Sx, Kz, Kx);
+        G2 = new_b(B2, E0, E1, J0, J1, Sx, Sy, Kx, Ky);
+        sx = fma_t(kx, F0.x, fma_t(ky, F1.x, kz * F2.x));
+        sy = fma_t(kx, F0.y, fma_t(ky, F1.y, kz * F2.y));
+    } else {
+        // Staggered components: E_a and J_a are p_a away from nodal position
+        // (p_a = exp(-i k_a/2), unit), B_a p_b p_c.  Shifted to it, advanced and
+        // shifted back, the phases meet khat only as kappa_a = khat_a p_a and its
+        // conjugate: e.g. conj(p_x) khat_y (p_x p_y B_z) = kappa_y B_z.
+        const cpx<T>* ph = a.tabc + d.tab_ph;
+        const cpx<T> px = ldg_c(ph + xp), py = ldg_c(ph + lxh + yp), pz = ldg_c(ph + lxh + Ly + zp);
+        const cpx<T> k0 = scale(px, hx), k1 = scale(py, hy), k2 = scale(pz, hz);
+        // acc + w v and acc + conj(w) v
+        auto mac = [](cpx<T> acc, cpx<T> w, cpx<T> v) {
+            return mk(fma_t(w.x, v.x, fma_t(-w.y, v.y, acc.x)), fma_t(w.x, v.y, fma_t(w.y, v.x, acc.y)));
+        };
+        auto macc = [](cpx<T> acc, cpx<T> w, cpx<T> v) {
+            return mk(fma_t(w.x, v.x, fma_t(w.y, v.y, acc.x)), fma_t(w.x, v.y, fma_t(-w.y, v.x, acc.y)));
+        };
+        auto ej = [&](cpx<T> E, cpx<T> J) { return mk(fma_t(omC, E.x, Dk * J.x), fma_t(omC, E.y, Dk * J.y)); };
+        const cpx<T> lo = mac(mac(cmul(k2, ej(E2, J2)), k1, ej(E1, J1)), k0, ej(E0, J0));
+        const cpx<T> is0 = mul_i(scale(k0, S)), is1 = mul_i(scale(k1, S)), is2 = mul_i(scale(k2, S));   // i S kappa
+        auto neg = [](cpx<T> v) { return mk(-v.x, -v.y); };
+        auto new_e = [&](cpx<T> Ea, cpx<T> Bb, cpx<T> Bc, cpx<T> Ja, cpx<T> ka, cpx<T> ib, cpx<T> ic) {
+            const cpx<T> v = mk(fma_t(C, Ea.x, -Sk * Ja.x), fma_t(C, Ea.y, -Sk * Ja.y));
+            return macc(mac(mac(v, ib, Bc), neg(ic), Bb), ka, lo);
+        };
+        // - i S conj(kappa) = conj(i S kappa);  i K conj(kappa) = -conj(i K kappa)
+        const cpx<T> ik0 = mul_i(scale(k0, omCk)), ik1 = mul_i(scale(k1, omCk)), ik2 = mul_i(scale(k2, omCk));
+        auto new_b = [&](cpx<T> Ba, cpx<T> Eb, cpx<T> Ec, cpx<T> Jb, cpx<T> Jc, cpx<T> ib, cpx<T> ic, cpx<T> jb, cpx<T> jc) {
+            return macc(macc(macc(macc(scale(Ba, C), ib, Ec), neg(ic), Eb), neg(jb), Jc), jc, Jb);
+        };
+        F0 = new_e(E0, B1, B2, J0, k0, is1, is2);
+        F1 = new_e(E1, B2, B0, J1, k1, is2, is0);
+        F2 = new_e(E2, B0, B1, J2, k2, is0, is1);
+        G0 = new_b(B0, E1, E2, J1, J2, is1, is2, ik1, ik2);
+        G1 = new_b(B1, E2, E0, J2, J0, is2, is0, ik2, ik0);
+        G2 = new_b(B2, E0, E1, J0, J1, is0, is1, ik0, ik1);
+        const cpx<T> s = mac(mac(cmul(scale(pz, kz), F2), scale(py, ky), F1), scale(px, kx), F0);
+        sx = s.x;
+        sy = s.y;
+    }
     if (nf > 9) {
-        // Gauss residual i[k].E' - rho on the unnormalised spectrum
+        // Gauss residual on the unnormalised spectrum: |i[k].E' N - rho|^2 =
+        // (N sy + rho_x)^2 + (N sx - rho_y)^2
         const cpx<T> rho = p[9 * fs];
-        const cpx<T> div = mul_i(scale(F0, kx) + scale(F1, ky) + scale(F2, kz));
-        const T rx = fma_t(div.x, Nfull, -rho.x);
-        const T ry = fma_t(div.y, Nfull, -rho.y);
+        const T rx = fma_t(sy, Nfull, rho.x);
+        const T ry = fma_t(sx, Nfull, -rho.y);
         const T wgt = (xp == 0 || xp == lxh - 1) ? T(1) : T(2);
         g_res += wgt * (rx * rx + ry * ry);
         g_rho += wgt * (rho.x * rho.x + rho.y * rho.y);
-    }
-    if (a.staggered) {
-        const cpx<T> pyz = cmul(py, pz), pxz = cmul(px, pz), pxy = cmul(px, py);
-        F0 = cmulc(F0, px); F1 = cmulc(F1, py); F2 = cmulc(F2, pz);
-        G0 = cmulc(G0, pyz); G1 = cmulc(G1, pxz); G2 = cmulc(G2, pxy);
     }
     p[0] = F0; p[fs] = F1; p[2 * fs] = F2;
     p[3 * fs] = G0; p[4 * fs] = G1; p[5 * fs] = G2;

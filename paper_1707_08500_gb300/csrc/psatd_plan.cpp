@@ -236,21 +236,30 @@ static int cuda_fail(psatd_plan_s* p, cudaError_t e, const char* where) {
 }
 
 // Device image of the twiddle pool: exp(-2 pi i m/n) per transform length and
-// the real-split twiddles exp(-2 pi i k/Lx) in position order.
+// half the real-split twiddles, exp(-2 pi i k/Lx)/2, in position order (the
+// split's factor 1/2; exact).
 static std::vector<char> twiddle_image(const psatd_plan_s* p) {
     std::vector<cd> tw(size_t(p->n_tw));
+    std::vector<char> half(size_t(p->n_tw), 0);
     for (auto& kv : p->tw_off)
         for (int m = 0; m < kv.first; ++m) tw[kv.second + m] = unit_root(m, kv.first);
     for (auto& kv : p->post_off) {
         const int Lx = kv.first / 32, f1 = kv.first % 32, h = Lx / 2;
-        for (int P = 0; P < h; ++P) tw[kv.second + P] = unit_root(axis_nat(h, f1, P), Lx);
+        for (int P = 0; P < h; ++P) {
+            tw[kv.second + P] = unit_root(axis_nat(h, f1, P), Lx);
+            half[size_t(kv.second) + P] = 1;
+        }
     }
     // each twiddle is stored as (hi, lo): in FP32 lo is the rounding of the
     // remainder so that hi + lo carries the FP64 value; in FP64 lo = 0
     std::vector<char> out;
     if (p->f64) {
         std::vector<double> t64(tw.size() * 4, 0.0);
-        for (size_t i = 0; i < tw.size(); ++i) { t64[4 * i] = tw[i].real(); t64[4 * i + 1] = tw[i].imag(); }
+        for (size_t i = 0; i < tw.size(); ++i) {
+            const double c = half[i] ? 0.5 : 1.0;
+            t64[4 * i] = c * tw[i].real();
+            t64[4 * i + 1] = c * tw[i].imag();
+        }
         out.assign(reinterpret_cast<const char*>(t64.data()), reinterpret_cast<const char*>(t64.data() + t64.size()));
     } else {
         std::vector<float> t32(tw.size() * 4);
@@ -261,6 +270,8 @@ static std::vector<char> twiddle_image(const psatd_plan_s* p) {
             t32[4 * i + 1] = hi;
             t32[4 * i + 2] = float(tw[i].real() - double(hr));
             t32[4 * i + 3] = float(tw[i].imag() - double(hi));
+            if (half[i])
+                for (int k = 0; k < 4; ++k) t32[4 * i + k] *= 0.5f;
         }
         out.assign(reinterpret_cast<const char*>(t32.data()), reinterpret_cast<const char*>(t32.data() + t32.size()));
     }
@@ -517,7 +528,7 @@ int psatd_plan_create_tuned(psatd_plan_t* out, const int32_t global_n[3], const 
     for (auto& d : p->desc) {
         for (AxisPlan* ap : {&d.ax, &d.ay, &d.az}) ap->tw = add_tw(ap->n);
     }
-    // real-split twiddles exp(-2 pi i k/Lx) stored in the position order of the
+    // halved real-split twiddles exp(-2 pi i k/Lx)/2 in the position order of the
     // x transform (entry P holds k = P/f2 + f1*(P%f2)), one table per (Lx, f1)
     for (auto& d : p->desc) {
         const int key = d.L[0] * 32 + d.ax.f1;   // (Lx, f1) fixes the split (axis_nat)

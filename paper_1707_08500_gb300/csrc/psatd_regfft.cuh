@@ -115,33 +115,10 @@ __device__ __forceinline__ void sts4(cpx<float>* p, cpx<float> a, cpx<float> b) 
 
 // ---- x: one row per thread -----------------------------------------------------
 // The twiddles come from the plan's pool: tw = exp(-2 pi i m/H), m = 0..H-1
-// (the axis table), wp = exp(-2 pi i k/Lx) for the frequency k at every
+// (the axis table), wp = exp(-2 pi i k/Lx)/2 for the frequency k at every
 // position of the packed transform (the real-split table); both as FP32
 // hi + lo pairs.  Outer loops run at run time so that the code of one length
 // stays small; the DFT bodies are unrolled.
-
-// Real split of one pair of positions of the packed transform: A = Z[pa],
-// B = Z[pb] (pb the partner of pa); X[pa] = e + w o, X[pb] = conj(e - w o)
-// with e = (A + conj B)/2, o = (A - conj B)/(2i), w the real-split twiddle of pa.
-__device__ __forceinline__ void split_pair_c(cpx<float> A, cpx<float> B, cpx<float> w, cpx<float>& outA,
-                                             cpx<float>& outB) {
-    const cpx<float> Bc = conj(B);
-    const cpx<float> e = scale(A + Bc, 0.5f);
-    const cpx<float> dd = A - Bc;
-    const cpx<float> wo = mul_tw(mk(0.5f * dd.y, -0.5f * dd.x), w);
-    outA = e + wo;
-    outB = conj(e - wo);
-}
-// Inverse of split_pair_c: X[pa] = A, X[pb] = B -> Z[pa] = e + i o,
-// Z[pb] = conj(e) + i conj(o), e = A + conj B, o = (A - conj B) conj(w).
-__device__ __forceinline__ void merge_pair_c(cpx<float> A, cpx<float> B, cpx<float> w, cpx<float>& outA,
-                                             cpx<float>& outB) {
-    const cpx<float> Bc = conj(B);
-    const cpx<float> e = A + Bc;
-    const cpx<float> o = mul_tw_conj(A - Bc, w);
-    outA = e + mul_i(o);
-    outB = conj(e) + mul_i(conj(o));
-}
 
 // Forward real transform of one row: row[0..H) holds z[m] = x[2m] + i x[2m+1]
 // (16-byte aligned); on return row[0..H) holds the half spectrum X[0..H) in
@@ -188,7 +165,7 @@ __device__ __forceinline__ void row_fwd(cpx<float>* row, const twd<float>* __res
 #pragma unroll
         for (int P = 1; P <= F2 / 2; ++P) {
             cpx<float> oa, ob;
-            split_pair_c(v[P], v[F2 - P], ld_tw(wp + P), oa, ob);
+            split_pair_v(v[P], v[F2 - P], ld_tw(wp + P), oa, ob);
             o[P] = oa;
             if (P != F2 - P) o[F2 - P] = ob;
         }
@@ -205,7 +182,7 @@ __device__ __forceinline__ void row_fwd(cpx<float>* row, const twd<float>* __res
 #pragma unroll
         for (int k2 = 0; k2 < F2; ++k2) {
             cpx<float> oa, ob;
-            split_pair_c(va[k2], vb[F2 - 1 - k2], ld_tw(wp + k1 * F2 + k2), oa, ob);
+            split_pair_v(va[k2], vb[F2 - 1 - k2], ld_tw(wp + k1 * F2 + k2), oa, ob);
             va[k2] = oa;
             vb[F2 - 1 - k2] = ob;
         }
@@ -222,7 +199,7 @@ __device__ __forceinline__ void row_fwd(cpx<float>* row, const twd<float>* __res
 #pragma unroll
         for (int k2 = 0; k2 < F2 / 2; ++k2) {
             cpx<float> oa, ob;
-            split_pair_c(v[k2], v[F2 - 1 - k2], ld_tw(wp + k1 * F2 + k2), oa, ob);
+            split_pair_v(v[k2], v[F2 - 1 - k2], ld_tw(wp + k1 * F2 + k2), oa, ob);
             v[k2] = oa;
             v[F2 - 1 - k2] = ob;
         }
@@ -257,7 +234,7 @@ __device__ __forceinline__ void row_inv(cpx<float>* row, const twd<float>* __res
 #pragma unroll
         for (int P = 1; P <= F2 / 2; ++P) {
             cpx<float> oa, ob;
-            merge_pair_c(v[P], v[F2 - P], ld_tw(wp + P), oa, ob);
+            merge_pair_v(v[P], v[F2 - P], ld_tw(wp + P), oa, ob);
             o[P] = oa;
             if (P != F2 - P) o[F2 - P] = ob;
         }
@@ -275,7 +252,7 @@ __device__ __forceinline__ void row_inv(cpx<float>* row, const twd<float>* __res
 #pragma unroll
         for (int k2 = 0; k2 < F2; ++k2) {
             cpx<float> oa, ob;
-            merge_pair_c(va[k2], vb[F2 - 1 - k2], ld_tw(wp + k1 * F2 + k2), oa, ob);
+            merge_pair_v(va[k2], vb[F2 - 1 - k2], ld_tw(wp + k1 * F2 + k2), oa, ob);
             va[k2] = oa;
             vb[F2 - 1 - k2] = ob;
         }
@@ -290,7 +267,7 @@ __device__ __forceinline__ void row_inv(cpx<float>* row, const twd<float>* __res
 #pragma unroll
         for (int k2 = 0; k2 < F2 / 2; ++k2) {
             cpx<float> oa, ob;
-            merge_pair_c(v[k2], v[F2 - 1 - k2], ld_tw(wp + k1 * F2 + k2), oa, ob);
+            merge_pair_v(v[k2], v[F2 - 1 - k2], ld_tw(wp + k1 * F2 + k2), oa, ob);
             v[k2] = oa;
             v[F2 - 1 - k2] = ob;
         }
