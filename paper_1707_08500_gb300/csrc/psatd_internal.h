@@ -48,6 +48,17 @@ constexpr int reg_pitch(int lxh) { return lxh + ((2 - lxh % 4) + 4) % 4; }
 constexpr int kZModes = 8, kZModesHeat = 16;
 constexpr int64_t kZMaxElems = int64_t(1) << 31;   // of a box's coefficient tables and of its spectra (32-bit offsets)
 
+// FP32 split-plane schedule and z stage with one axis length compiled in (every
+// box of the plan has it, at its default split): the x lengths of the row
+// launches, the y lengths of the column launches (kSplitCols columns an item),
+// and the z lengths with their modes per item (long axes take fewer, so that
+// two or three blocks share an SM's shared memory).
+constexpr int kSplitCols = 16;
+constexpr int kSplitX[] = {128, 192, 256, 384, 512};
+constexpr int kSplitY[] = {128, 192, 256};
+struct ZChunk { int L, M; };
+constexpr ZChunk kLongZ[] = {{128, 8}, {192, 4}, {256, 4}};
+
 // Cubic local boxes (side L, ng guards, pass-B chunk M, default splits) that
 // have kernels compiled with their geometry fixed at compile time.
 struct FixedGeo { int L, ng, M; };
@@ -128,6 +139,7 @@ struct LaunchCommon {
     int nout;             // output fields written by the inverse stages: 6 (E, B) or 1 (heat: T)
     int64_t per_sub[5];   // items per subdomain of passes A, B, C and of the split schedule's column stages
                           // (forward, inverse) when every subdomain has the same shape, else 0
+    int splitX, splitY, longZ;   // axis lengths compiled in (kSplitX, kSplitY, kLongZ), or 0
     int variant;          // index into kFixedF32 / kFixedF64, or -1 for the descriptor-driven kernels
 };
 

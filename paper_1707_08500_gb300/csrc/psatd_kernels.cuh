@@ -689,6 +689,42 @@ __device__ __forceinline__ void store_plane(const Args<T>& a, const SubDesc& d, 
     }
 }
 
+// Run-time geometry with one axis fixed at compile time (0: none): the x length
+// of the row launches of the split-plane schedule, the y length of its column
+// launches, the z length and the chunk width of the z stage.
+template <int LX>
+struct GeoRows : GeoDyn {
+    static constexpr bool kThree = LX == 0;
+    static constexpr int kH = LX / 2;
+    __device__ explicit GeoRows(const SubDesc& d) : GeoDyn(d) {
+        if constexpr (LX > 0) {
+            h = kH; lxh = kH + 1; pitch = (kH + 1) | 1;
+            ax = AxisPlan{kH, split_first(kH), kH / split_first(kH), d.ax.tw, 0, 0};
+        }
+    }
+};
+template <int LY>
+struct GeoCols : GeoDyn {
+    static constexpr bool kThree = LY == 0;
+    __device__ explicit GeoCols(const SubDesc& d) : GeoDyn(d) {
+        if constexpr (LY > 0) {
+            Ly = LY;
+            ay = AxisPlan{LY, split_first(LY), LY / split_first(LY), d.ay.tw, 0, 0};
+        }
+    }
+};
+template <int LZ, int MB>
+struct GeoZ {
+    static constexpr bool kFixed = false;
+    static constexpr bool kThree = false;
+    static constexpr int M = MB, lgM = (MB & (MB - 1)) ? -1 : ilog2(MB), Lz = LZ, fs = pad_field_stride(LZ, MB, 8);
+    int Lx, Ly, h, lxh, pitch, q, ng, ngz, nvy, nvz;
+    AxisPlan ax, ay, az;
+    __device__ explicit GeoZ(const SubDesc& d)
+        : Lx(d.L[0]), Ly(d.L[1]), h(d.L[0] >> 1), lxh(d.lxh), pitch(d.pitch), q(d.q), ng(d.ng), ngz(d.ngz), nvy(d.nv[1]),
+          nvz(d.nv[2]), ax(d.ax), ay(d.ay), az{LZ, split_first(LZ), LZ / split_first(LZ), d.az.tw, 0, 0} {}
+};
+
 // ---- pass A: x (real) and y forward transforms of one plane ---------------
 template <typename T, class G>
 __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? (G::kFixed ? PSATD_MINB_A_FIXED : PSATD_MINB_A) : 2)
@@ -1085,7 +1121,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? PSATD_MINB_C : 2) k
 // then stage 7 (real merge, x rows, the exchange scatter of pass C).
 
 // stage 4: x (real) transforms of a block of rows of one input plane
-template <typename T>
+template <typename T, int LX = 0>
 __global__ void __launch_bounds__(kThreads) k_rows_fwd(Args<T> a) {
     extern __shared__ __align__(16) unsigned char smraw[];
     cpx<T>* sm = reinterpret_cast<cpx<T>*>(smraw);
@@ -1095,7 +1131,7 @@ __global__ void __launch_bounds__(kThreads) k_rows_fwd(Args<T> a) {
     for (int64_t it = tk.current(); it >= 0; tk.advance(), it = tk.current()) {
         tk.prefetch();
         decode_item<4>(a, it, &d);
-        const GeoDyn g(d);
+        const GeoRows<LX> g(d);
         const int R = d.rows, nb = (g.Ly + R - 1) / R;
         const int loc = int(it - d.itemA);
         const int pl = loc / nb, rb = loc - pl * nb;
@@ -1107,7 +1143,7 @@ __global__ void __launch_bounds__(kThreads) k_rows_fwd(Args<T> a) {
         loop2(h, nr, [&](int y, int m) { cp_async_c(sm + y * pitch + m, src + y * h + m); });
         cp_async_wait_all();
         __syncthreads();
-        fft_fwd<false>(sm, g.ax, Batch{nr, pitch, 0, 0, 1, 1}, a.tw);
+        fft_fwd<false, T, GeoRows<LX>::kThree>(sm, g.ax, Batch{nr, pitch, 0, 0, 1, 1}, a.tw);
         real_split_rows(sm, nr, pitch, h, g.ax, a.tw + d.tw_post);
         __syncthreads();
         cpx<T>* dst = a.spec + d.spec_off + int64_t(f * g.Lz + z) * g.q + int64_t(y0) * lxh;
@@ -1119,7 +1155,7 @@ __global__ void __launch_bounds__(kThreads) k_rows_fwd(Args<T> a) {
 // stages 5 (forward, every plane of the nf input fields) and 6 (inverse, the
 // valid z planes of the six outputs): y transforms of `cols` columns of one
 // plane; the inverse stores only the valid rows, the only ones stage 7 reads
-template <typename T, bool INV>
+template <typename T, bool INV, int LY = 0>
 __global__ void __launch_bounds__(kThreads) k_cols(Args<T> a) {
     extern __shared__ __align__(16) unsigned char smraw[];
     cpx<T>* sm = reinterpret_cast<cpx<T>*>(smraw);
@@ -1129,8 +1165,8 @@ __global__ void __launch_bounds__(kThreads) k_cols(Args<T> a) {
     for (int64_t it = tk.current(); it >= 0; tk.advance(), it = tk.current()) {
         tk.prefetch();
         decode_item<INV ? 6 : 5>(a, it, &d);
-        const GeoDyn g(d);
-        const int W = d.cols, lxh = g.lxh, Ly = g.Ly, nb = (lxh + W - 1) / W;
+        const GeoCols<LY> g(d);
+        const int W = LY ? kSplitCols : d.cols, lxh = g.lxh, Ly = g.Ly, nb = (lxh + W - 1) / W;
         const int loc = int(it - (INV ? d.itemC1 : d.itemA2));
         const int pl = loc / nb, cb = loc - pl * nb;
         int f, z;
@@ -1145,8 +1181,8 @@ __global__ void __launch_bounds__(kThreads) k_cols(Args<T> a) {
         });
         cp_async_wait_all();
         __syncthreads();
-        if constexpr (INV) fft_inv<false>(sm, g.ay, Batch{W, 1, 0, 0, W, 1}, a.tw);
-        else fft_fwd<false>(sm, g.ay, Batch{W, 1, 0, 0, W, 1}, a.tw);
+        if constexpr (INV) fft_inv<false, T, GeoCols<LY>::kThree>(sm, g.ay, Batch{W, 1, 0, 0, W, 1}, a.tw);
+        else fft_fwd<false, T, GeoCols<LY>::kThree>(sm, g.ay, Batch{W, 1, 0, 0, W, 1}, a.tw);
         const int ya = INV ? g.ng : 0, ny = INV ? g.nvy : Ly;
         loop2(W, ny, [&](int y, int m) {
             if (m < wc) stcs_c(base + int64_t(ya + y) * lxh + m, sm[(ya + y) * W + m]);
@@ -1157,7 +1193,7 @@ __global__ void __launch_bounds__(kThreads) k_cols(Args<T> a) {
 
 // stage 7: real merge and inverse x transforms of a block of valid rows of one
 // output plane, then the store of pass C (own box and every guard image)
-template <typename T>
+template <typename T, int LX = 0>
 __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? PSATD_MINB_ROWS : 2) k_rows_inv(Args<T> a) {
     extern __shared__ __align__(16) unsigned char smraw[];
     cpx<T>* sm = reinterpret_cast<cpx<T>*>(smraw);
@@ -1168,7 +1204,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? PSATD_MINB_ROWS : 2
     for (int64_t it = tk.current(); it >= 0; tk.advance(), it = tk.current()) {
         tk.prefetch();
         decode_item<7>(a, it, &d);
-        const GeoDyn g(d);
+        const GeoRows<LX> g(d);
         const int R = d.rows, nb = (g.nvy + R - 1) / R;
         const int loc = int(it - d.itemC);
         const int pl = loc / nb, rb = loc - pl * nb;
@@ -1183,7 +1219,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? PSATD_MINB_ROWS : 2
         __syncthreads();
         real_merge_rows(sm, nr, pitch, h, g.ax, a.tw + d.tw_post);
         __syncthreads();
-        fft_inv<false>(sm, g.ax, Batch{nr, pitch, 0, 0, 1, 1}, a.tw);
+        fft_inv<false, T, GeoRows<LX>::kThree>(sm, g.ax, Batch{nr, pitch, 0, 0, 1, 1}, a.tw);
         store_plane<kThreads>(a, d, z, ya, ya + nr, ya, rs, &plan, kThreads / 32 - 1, a.eb[f], reinterpret_cast<const T*>(sm));
         __syncthreads();
     }

@@ -23,6 +23,7 @@ cudaError_t launch_stage_f64(int stage, const LaunchCommon& c, int64_t i0, int64
 cudaError_t launch_gauss_reduce(const void* subs, int nsub, const double* part, double* out, cudaStream_t st);
 cudaError_t launch_stage_reg(int stage, int rows, const LaunchCommon& c, int64_t i0, int64_t n, int smem, cudaStream_t s);
 cudaError_t launch_stage_z(int zlen, bool heat, bool stag, const LaunchCommon& c, int64_t i0, int64_t n, int smem, cudaStream_t s);
+bool launch_stage_length(int stage, const LaunchCommon& c, int64_t i0, int64_t n, int smem, cudaStream_t s, cudaError_t* err);
 cudaError_t launch_stage_flat(bool stag, const LaunchCommon& c, int64_t i0, int64_t n, cudaStream_t s);
 }  // namespace psatd
 
@@ -206,6 +207,7 @@ struct psatd_plan_s {
     bool reg = false;                  // FP32 plane stages with compile-time-length transforms
     bool regB = false;                 // PSATD_PACKED_Z honoured (reported by psatd_plane_engine)
     bool zpass = false;                // FP32 z stage of psatd_zpass.cuh (else the generic one)
+    int splitX = 0, splitY = 0, longZ = 0;   // FP32 axis lengths compiled in (split-plane schedule, z stage)
     bool flat = false;                 // FP32, every box one cell deep: Eq. 1 without a z transform
     int zlen = 0;                      // its z length when every box has the same, else 0
     int smemAreg = 0, smemCreg = 0, regRows = 0;
@@ -586,6 +588,17 @@ int psatd_plan_create_tuned(psatd_plan_t* out, const int32_t global_n[3], const 
         p->regB = (flags & PSATD_PACKED_Z) && set && even && !p->heat && (!asked || asked == 6);
         p->zpass = p->regB || (set && (p->heat || (same && !p->stag)) && (!asked || asked == (p->heat ? kZModesHeat : kZModes)));
         p->zlen = same ? d0.L[2] : 0;
+        // axes of one compiled length in every box (kSplitX, kSplitY, kLongZ) at
+        // their default splits
+        bool sx = true, sy = true, sz = !p->heat && !asked;
+        for (const SubDesc& d : p->desc) {
+            sx = sx && d.L[0] == d0.L[0] && d.ax.f3 <= 1 && d.ax.f1 == split_first(d.L[0] / 2);
+            sy = sy && d.L[1] == d0.L[1] && d.ay.f3 <= 1 && d.ay.f1 == split_first(d.L[1]) && d.lxh >= kSplitCols;
+            sz = sz && d.L[2] == d0.L[2] && d.az.f3 <= 1 && d.az.f1 == split_first(d.L[2]);
+        }
+        for (int v : kSplitX) if (sx && d0.L[0] == v) p->splitX = v;
+        for (int v : kSplitY) if (sy && d0.L[1] == v) p->splitY = v;
+        for (const ZChunk& v : kLongZ) if (sz && d0.L[2] == v.L) p->longZ = v.L;
         // boxes one cell deep (2D problems) take Eq. 1 alone, for any chunk
         p->flat = !p->heat;
         for (const SubDesc& d : p->desc) p->flat = p->flat && d.L[2] == 1 && TAB_N * int64_t(d.q) < kZMaxElems;
@@ -600,6 +613,7 @@ int psatd_plan_create_tuned(psatd_plan_t* out, const int32_t global_n[3], const 
             while (M < 64 && int64_t(p->nf) * d.L[2] * (2 * M) * csz <= 32 * 1024) M *= 2;
         while (M > 1 && int64_t(p->nf) * (d.L[2] * M + 16) * csz > 200 * 1024) M /= 2;
         if (p->zpass) M = p->heat ? kZModesHeat : kZModes;
+        for (const ZChunk& v : kLongZ) if (p->longZ == v.L) M = v.M;
         d.chunkB = M;
         d.lgB = 0;
         while ((1 << d.lgB) < M) ++d.lgB;
@@ -635,7 +649,7 @@ int psatd_plan_create_tuned(psatd_plan_t* out, const int32_t global_n[3], const 
         d.cols = d.lxh;
         if (p->split) {
             d.rows = std::max(1, std::min(d.L[1], kSplitRowBytes / (d.pitch * csz)));
-            d.cols = std::min(d.lxh, p->f64 ? 8 : 16);
+            d.cols = std::min(d.lxh, p->f64 ? 8 : kSplitCols);
             d.itemA2 = iA2; d.itemC1 = iC1;
             const int64_t rb_in = (d.L[1] + d.rows - 1) / d.rows, rb_out = (d.nv[1] + d.rows - 1) / d.rows;
             const int64_t cb = (d.lxh + d.cols - 1) / d.cols;
@@ -684,7 +698,7 @@ int psatd_plan_create_tuned(psatd_plan_t* out, const int32_t global_n[3], const 
     if (p->variant < 0 && !p->split) {
         bool dflt = true;
         for (const SubDesc& d : p->desc)
-            dflt = dflt && (d.chunkB == (p->f64 ? 4 : 8) || (p->zpass && !p->heat)) && d.ax.f3 <= 1 && d.ay.f3 <= 1 && d.az.f3 <= 1;
+            dflt = dflt && (d.chunkB == (p->f64 ? 4 : 8) || (p->zpass && !p->heat) || p->longZ) && d.ax.f3 <= 1 && d.ay.f3 <= 1 && d.az.f3 <= 1;
         if (dflt) p->variant = -2;
     }
     if (p->smemB > kPlaneSmemMax || (p->split && std::max(p->smemR, p->smemK) > kPlaneSmemMax))
@@ -1026,6 +1040,9 @@ static LaunchCommon common_at(psatd_plan_s* p, char* base, const psatd_fields* f
     c.staggered = p->stag ? 1 : 0;
     c.own_only = 0;
     for (int i = 0; i < 5; ++i) c.per_sub[i] = p->per_sub[i];
+    c.splitX = p->splitX;
+    c.splitY = p->splitY;
+    c.longZ = p->longZ;
     c.variant = p->variant;
     return c;
 }
@@ -1033,6 +1050,8 @@ static LaunchCommon common_at(psatd_plan_s* p, char* base, const psatd_fields* f
 static LaunchCommon common(psatd_plan_s* p, const psatd_fields* f) { return common_at(p, p->ws, f); }
 
 static cudaError_t stage(psatd_plan_s* p, int st, const LaunchCommon& c, int64_t i0, int64_t n, int smem, cudaStream_t s) {
+    cudaError_t e;
+    if (!p->f64 && launch_stage_length(st, c, i0, n, smem, s, &e)) return e;
     return p->f64 ? launch_stage_f64(st, c, i0, n, smem, s) : launch_stage_f32(st, c, i0, n, smem, s);
 }
 

@@ -1,0 +1,44 @@
+// FP32 stages with one axis length compiled in: the row and column launches of
+// the split-plane schedule and the z stage of long axes (one box over the grid,
+// the global solver).  With the geometry read at run time these kernels spend
+// their issue slots on index arithmetic and hold 80 registers; a 256^3 box:
+// forward launches 850 to 700 us, z stage 660 to 573 (four modes an item and two
+// blocks per SM instead of eight and one), inverse launches 543 to 474.
+#include "psatd_kernels.cuh"
+
+namespace psatd {
+
+// f(integral_constant) for v among the lengths of `list`
+template <const auto& list, int I = 0, class F>
+static bool with_length(int v, F&& f) {
+    if constexpr (I < int(sizeof(list) / sizeof(list[0]))) {
+        if (v == list[I]) { f(std::integral_constant<int, list[I]>{}); return true; }
+        return with_length<list, I + 1>(v, f);
+    }
+    return false;
+}
+
+// Stages 1 and 4 to 7 (see stage_item); false when the plan's length is not
+// compiled in.
+bool launch_stage_length(int stage, const LaunchCommon& c, int64_t item0, int64_t nitems, int smem, cudaStream_t st,
+                         cudaError_t* err) {
+    *err = cudaSuccess;
+    const Args<float> a = make_args<float>(c, item0, nitems);
+    auto go = [&](auto k) { if (nitems > 0) *err = launch_kernel<float>(k, a, smem, st); };
+    if (stage == 1) {
+        if (c.longZ == 128) go(k_pass_b<float, GeoZ<kLongZ[0].L, kLongZ[0].M>>);
+        else if (c.longZ == 192) go(k_pass_b<float, GeoZ<kLongZ[1].L, kLongZ[1].M>>);
+        else if (c.longZ == 256) go(k_pass_b<float, GeoZ<kLongZ[2].L, kLongZ[2].M>>);
+        else return false;
+        return true;
+    }
+    switch (stage) {
+        case 4: return with_length<kSplitX>(c.splitX, [&](auto l) { go(k_rows_fwd<float, decltype(l)::value>); });
+        case 5: return with_length<kSplitY>(c.splitY, [&](auto l) { go(k_cols<float, false, decltype(l)::value>); });
+        case 6: return with_length<kSplitY>(c.splitY, [&](auto l) { go(k_cols<float, true, decltype(l)::value>); });
+        case 7: return with_length<kSplitX>(c.splitX, [&](auto l) { go(k_rows_inv<float, decltype(l)::value>); });
+        default: return false;
+    }
+}
+
+}  // namespace psatd
