@@ -24,8 +24,7 @@ cudaError_t launch_stage_f32(int stage, const LaunchCommon& c, int64_t item0, in
 cudaError_t launch_gauss_reduce(const void* subs, int nsub, const double* part, double* out, cudaStream_t st) {
     const int threads = 256;
     const int blocks = (nsub * 32 + threads - 1) / threads;
-    k_gauss_reduce<<<blocks, threads, 0, st>>>(static_cast<const SubDesc*>(subs), nsub, part, out);
-    return cudaPeekAtLastError();
+    return launch_overlapped(k_gauss_reduce, unsigned(blocks), threads, 0, st, static_cast<const SubDesc*>(subs), nsub, part, out);
 }
 
 }  // namespace psatd

@@ -1,9 +1,6 @@
 // FP32 stages with one axis length compiled in: the row and column launches of
 // the split-plane schedule and the z stage of long axes (one box over the grid,
-// the global solver).  With the geometry read at run time these kernels spend
-// their issue slots on index arithmetic and hold 80 registers; a 256^3 box:
-// forward launches 850 to 700 us, z stage 660 to 573 (four modes an item and two
-// blocks per SM instead of eight and one), inverse launches 543 to 474.
+// the global solver).
 #include "psatd_kernels.cuh"
 
 namespace psatd {

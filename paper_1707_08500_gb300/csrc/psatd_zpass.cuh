@@ -192,6 +192,7 @@ __global__ void __launch_bounds__(NW * 32, MINB) k_pass_z(Args<float> a) {
     __shared__ cpx<float> s_tw[CN ? 4 * CN : 96];   // w^(j r) at j N + r, j < 4, r < N
     const int warp = int(threadIdx.x) >> 5, lane = int(threadIdx.x) & 31;
     const TicketDraw<float> draw{a};
+    wait_for_previous_launch();
     if (threadIdx.x == 0) {
         s_it[0] = draw.first();
         s_it[1] = s_it[0] >= 0 ? draw.next() : -1;
