@@ -25,6 +25,7 @@
 
 #include "psatd.h"
 #include "psatd_fdtd.h"
+#include "psatd_launch.cuh"
 
 namespace {
 
@@ -109,6 +110,7 @@ __global__ void __launch_bounds__(NT) k_yee(YeeArgs<T> a) {
     constexpr int KE = (NIE + NT - 1) / NT, KB = (NIB + NT - 1) / NT, KJ = (NIJ + NT - 1) / NT;
     extern __shared__ __align__(16) unsigned char smraw[];
     L& s = *reinterpret_cast<L*>(smraw);
+    psatd::wait_for_previous_launch();
     const int t = threadIdx.x;
     const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY;
     const int z0 = blockIdx.z * KZ, z1 = min(z0 + KZ, a.nz);
@@ -331,8 +333,7 @@ int launch(const int32_t n[3], double c_dt, const double dx[3], const psatd_fiel
     auto k = fast ? k_yee<T, true> : k_yee<T, false>;
     if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess)
         return PSATD_E_CUDA;
-    k<<<grid, NT, smem, st>>>(a);
-    return cudaPeekAtLastError() == cudaSuccess ? PSATD_OK : PSATD_E_CUDA;
+    return psatd::launch_overlapped(k, grid, NT, smem, st, a) == cudaSuccess ? PSATD_OK : PSATD_E_CUDA;
 }
 
 }  // namespace

@@ -13,6 +13,7 @@
 #include <cstdint>
 
 #include "psatd_io.h"
+#include "psatd_launch.cuh"
 
 namespace psatd {
 
@@ -65,6 +66,7 @@ __device__ __forceinline__ void copy_rows(const VT* __restrict__ in, int64_t ild
 
 template <typename T>
 __global__ void __launch_bounds__(kIoThreads) k_scatter(IoArgs a) {
+    wait_for_previous_launch();
     const int64_t item = blockIdx.x;
     const int f = int(item / a.planes_local);
     const int64_t p = item - int64_t(f) * a.planes_local;
@@ -88,6 +90,7 @@ __global__ void __launch_bounds__(kIoThreads) k_scatter(IoArgs a) {
 
 template <typename T>
 __global__ void __launch_bounds__(kIoThreads) k_gather(IoArgs a) {
+    wait_for_previous_launch();
     const int64_t item = blockIdx.x;
     const int f = int(item / a.planes_valid);
     const int64_t p = item - int64_t(f) * a.planes_valid;
@@ -113,14 +116,8 @@ cudaError_t launch_io(bool scatter, bool f64, const IoArgs& a, cudaStream_t st) 
     if (items <= 0) return cudaSuccess;
     if (items > 2147483647) return cudaErrorInvalidConfiguration;
     const unsigned grid = unsigned(items);
-    if (scatter) {
-        if (f64) k_scatter<double><<<grid, kIoThreads, 0, st>>>(a);
-        else k_scatter<float><<<grid, kIoThreads, 0, st>>>(a);
-    } else {
-        if (f64) k_gather<double><<<grid, kIoThreads, 0, st>>>(a);
-        else k_gather<float><<<grid, kIoThreads, 0, st>>>(a);
-    }
-    return cudaPeekAtLastError();
+    void (*const k)(IoArgs) = scatter ? (f64 ? k_scatter<double> : k_scatter<float>) : (f64 ? k_gather<double> : k_gather<float>);
+    return launch_overlapped(k, dim3(grid), kIoThreads, 0, st, a);
 }
 
 }  // namespace psatd

@@ -25,6 +25,7 @@
 #include <stdint.h>
 
 #include "psatd_internal.h"
+#include "psatd_launch.cuh"
 #include "small_dft.cuh"
 
 #include <mutex>
@@ -508,16 +509,6 @@ __device__ __forceinline__ const T* field_in(const Args<T>& a, int f) {
 // workspace is attached).  Otherwise CTA b processes item item0 + b only.
 // Every loop body ends with __syncthreads(), which orders the slot writes and
 // reads.
-
-// Launches of one stream overlap at their ends: every stage kernel lets the next
-// one start its blocks as soon as slots free up (launch_dependents), and none
-// reads or writes global memory, the ticket counter included, before the
-// kernels ahead of it have finished and their writes are visible (wait).  Both
-// do nothing in a launch without the attribute.
-__device__ __forceinline__ void wait_for_previous_launch() {
-    asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
-    asm volatile("griddepcontrol.wait;\n" ::: "memory");
-}
 
 template <typename T>
 struct TicketDraw {
@@ -1350,26 +1341,6 @@ static cudaError_t launch_shape(const void* fn, int smem, bool persistent, int* 
     }
     *resident = (c->per_sm > 0 ? c->per_sm : 1) * c->nsm;
     return cudaSuccess;
-}
-
-// Launch that may start before the kernels ahead of it on the stream have
-// finished (see wait_for_previous_launch): a push is three to six dependent
-// launches, and their gaps and block start-up are what small problems wait for.
-// Eight boxes of 48^3: 97 to 86 us a step, one box of 32^3 63.5 to 60.9.
-template <class K, class... A>
-static cudaError_t launch_overlapped(K k, unsigned grid, int threads, int smem, cudaStream_t st, const A&... args) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(unsigned(threads));
-    cfg.dynamicSmemBytes = size_t(smem);
-    cfg.stream = st;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    const cudaError_t e = cudaLaunchKernelEx(&cfg, k, args...);
-    return e != cudaSuccess ? e : cudaPeekAtLastError();
 }
 
 // One launch of kernel k: persistent (as many CTAs as can be resident, each

@@ -1,0 +1,37 @@
+#pragma once
+// Launches that overlap at their ends.
+#include <cuda_runtime.h>
+
+namespace psatd {
+
+// Launches of one stream overlap at their ends: every kernel lets the next
+// one start its blocks as soon as slots free up (launch_dependents), and none
+// reads or writes global memory, the ticket counter included, before the
+// kernels ahead of it have finished and their writes are visible (wait).  Both
+// do nothing in a launch without the attribute.
+__device__ __forceinline__ void wait_for_previous_launch() {
+    asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
+    asm volatile("griddepcontrol.wait;\n" ::: "memory");
+}
+
+// Launch that may start before the kernels ahead of it on the stream have
+// finished (see wait_for_previous_launch): a push is three to six dependent
+// launches, and their gaps and block start-up are what small problems wait for.
+// Eight boxes of 48^3: 97 to 86 us a step, one box of 32^3 63.5 to 60.9.
+template <class K, class... A>
+static cudaError_t launch_overlapped(K k, dim3 grid, int threads, int smem, cudaStream_t st, const A&... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(unsigned(threads));
+    cfg.dynamicSmemBytes = size_t(smem);
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, k, args...);
+    return e != cudaSuccess ? e : cudaPeekAtLastError();
+}
+
+}  // namespace psatd
