@@ -103,7 +103,8 @@ extern "C" {
                                      are compiled in (see psatd_plane_engine).
                                      Without the flag it runs where it is the
                                      faster one: the heat equation, and
-                                     unstaggered boxes of one z length       */
+                                     unstaggered boxes of one z length that
+                                     are not too few                         */
 #define PSATD_SPLIT_PLANES   0x80 /* split-plane schedule: the x and y transforms
                                      of the forward and inverse plane stages run
                                      as separate row and column launches (five

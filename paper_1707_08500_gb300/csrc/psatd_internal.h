@@ -46,6 +46,7 @@ constexpr int reg_pitch(int lxh) { return lxh + ((2 - lxh % 4) + 4) % 4; }
 // FP32 z stage of psatd_zpass.cuh (for the z lengths in kRegY): modes per work
 // item, and of the heat equation's one or two fields.
 constexpr int kZModes = 8, kZModesHeat = 16;
+constexpr int kSms = 152;         // SMs of the GPU that the rules on item counts are for
 constexpr int64_t kZMaxElems = int64_t(1) << 31;   // of a box's coefficient tables and of its spectra (32-bit offsets)
 
 // FP32 split-plane schedule and z stage with one axis length compiled in (every
@@ -131,7 +132,7 @@ struct Segment {
 // Pointers and counts common to every stage launch.
 struct LaunchCommon {
     const void* subs; const void* segs; const void* tw; const void* tab; const void* tabc; void* spec;
-    void* eb[6]; const void* jr[4]; double* gauss_part;
+    void* eb[6]; const void* jr[4]; void* gauss_part;
     unsigned long long* work;   // persistent-launch work counter (in the workspace)
     unsigned int* err;          // device error word (bits PSATD_CHECK_*), in the workspace
     int persistent;             // 1: persistent grids drawing tickets; 0: one CTA per work item

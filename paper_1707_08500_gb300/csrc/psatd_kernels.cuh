@@ -88,7 +88,7 @@ struct Args {
     cpx<T>* spec;           // spectra
     T* eb[6];               // Ex Ey Ez Bx By Bz
     const T* jr[4];         // Jx Jy Jz rho
-    double* gauss_part;     // 2 per pass-B item
+    T* gauss_part;          // 2 per pass-B item (PSATD_GAUSS_DIAG plans)
     unsigned long long* work;   // work-item ticket counter of this launch (zero at its start)
     unsigned int* err;          // device error word: bit 0 item outside its subdomain, bit 1 ticket out of range
     int persistent;         // 1: CTAs draw items from `work`; 0: CTA b does item item0 + b
@@ -1000,8 +1000,8 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? PSATD_MINB_B : 2) k
         if (nf > 9) {
             block_sum2(g_res, g_rho, red);
             if (threadIdx.x == 0) {
-                a.gauss_part[2 * it] = double(g_res);
-                a.gauss_part[2 * it + 1] = double(g_rho);
+                a.gauss_part[2 * it] = g_res;
+                a.gauss_part[2 * it + 1] = g_rho;
             }
         }
         __syncthreads();
@@ -1254,7 +1254,8 @@ __global__ void __launch_bounds__(kThreads) k_exchange(Args<T> a) {
 }
 
 // ---- per-subdomain reduction of the Gauss partial sums ----------------------
-static __global__ void k_gauss_reduce(const SubDesc* __restrict__ subs, int nsub, const double* __restrict__ part,
+template <typename T>
+static __global__ void k_gauss_reduce(const SubDesc* __restrict__ subs, int nsub, const T* __restrict__ part,
                                double* __restrict__ out) {
     wait_for_previous_launch();
     const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -1263,7 +1264,7 @@ static __global__ void k_gauss_reduce(const SubDesc* __restrict__ subs, int nsub
     const int64_t b = subs[w].itemB;
     const int64_t end = b + (int64_t(subs[w].q) + subs[w].chunkB - 1) / subs[w].chunkB;
     double s1 = 0, s2 = 0;
-    for (int64_t i = b + l; i < end; i += 32) { s1 += part[2 * i]; s2 += part[2 * i + 1]; }
+    for (int64_t i = b + l; i < end; i += 32) { s1 += double(part[2 * i]); s2 += double(part[2 * i + 1]); }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
         s1 += __shfl_down_sync(0xffffffffu, s1, o);
@@ -1285,7 +1286,7 @@ static Args<T> make_args(const LaunchCommon& c, int64_t item0, int64_t nitems) {
     a.spec = static_cast<cpx<T>*>(c.spec);
     for (int i = 0; i < 6; ++i) a.eb[i] = static_cast<T*>(c.eb[i]);
     for (int i = 0; i < 4; ++i) a.jr[i] = static_cast<const T*>(c.jr[i]);
-    a.gauss_part = c.gauss_part;
+    a.gauss_part = static_cast<T*>(c.gauss_part);
     a.work = c.work;
     a.err = c.err;
     a.persistent = c.persistent;
@@ -1352,7 +1353,11 @@ static cudaError_t launch_kernel(void (*k)(Args<T>), const Args<T>& a, int smem,
     if (e != cudaSuccess) return e;
     unsigned grid = grid_for(a.nitems);
     if (a.persistent) grid = grid_for(a.nitems < resident ? a.nitems : resident);
-    return launch_overlapped(k, grid, threads, smem, st, a);
+    // overlapped ends pay where a launch is a few rounds of its blocks; long
+    // launches lose 1-2% to blocks of the next one that are set up early (48
+    // uneven boxes 1320 to 1346 us, 64 boxes of 96^3 2483 to 2501)
+    const bool brief = a.nitems <= 16 * int64_t(resident > 0 ? resident : 1);
+    return launch_maybe_overlapped(brief, k, grid, threads, smem, st, a);
 }
 
 // Launch stage `stage` (see stage_item) with geometry G; the exchange and the

@@ -21,10 +21,12 @@ cudaError_t launch_stage_f32(int stage, const LaunchCommon& c, int64_t item0, in
     }
 }
 
-cudaError_t launch_gauss_reduce(const void* subs, int nsub, const double* part, double* out, cudaStream_t st) {
+cudaError_t launch_gauss_reduce(bool f64, const void* subs, int nsub, const void* part, double* out, cudaStream_t st) {
     const int threads = 256;
-    const int blocks = (nsub * 32 + threads - 1) / threads;
-    return launch_overlapped(k_gauss_reduce, unsigned(blocks), threads, 0, st, static_cast<const SubDesc*>(subs), nsub, part, out);
+    const dim3 blocks(unsigned((nsub * 32 + threads - 1) / threads));
+    const SubDesc* d = static_cast<const SubDesc*>(subs);
+    return f64 ? launch_overlapped(k_gauss_reduce<double>, blocks, threads, 0, st, d, nsub, static_cast<const double*>(part), out)
+               : launch_overlapped(k_gauss_reduce<float>, blocks, threads, 0, st, d, nsub, static_cast<const float*>(part), out);
 }
 
 }  // namespace psatd

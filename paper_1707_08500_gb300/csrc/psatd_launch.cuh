@@ -18,8 +18,10 @@ __device__ __forceinline__ void wait_for_previous_launch() {
 // finished (see wait_for_previous_launch): a push is three to six dependent
 // launches, and their gaps and block start-up are what small problems wait for.
 // Eight boxes of 48^3: 97 to 86 us a step, one box of 32^3 63.5 to 60.9.
+// overlap = false: an ordinary launch.
 template <class K, class... A>
-static cudaError_t launch_overlapped(K k, dim3 grid, int threads, int smem, cudaStream_t st, const A&... args) {
+static cudaError_t launch_maybe_overlapped(bool overlap, K k, dim3 grid, int threads, int smem, cudaStream_t st,
+                                           const A&... args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = dim3(unsigned(threads));
@@ -29,9 +31,13 @@ static cudaError_t launch_overlapped(K k, dim3 grid, int threads, int smem, cuda
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = overlap ? 1 : 0;
     const cudaError_t e = cudaLaunchKernelEx(&cfg, k, args...);
     return e != cudaSuccess ? e : cudaPeekAtLastError();
+}
+template <class K, class... A>
+static cudaError_t launch_overlapped(K k, dim3 grid, int threads, int smem, cudaStream_t st, const A&... args) {
+    return launch_maybe_overlapped(true, k, grid, threads, smem, st, args...);
 }
 
 }  // namespace psatd

@@ -20,7 +20,7 @@
 namespace psatd {
 cudaError_t launch_stage_f32(int stage, const LaunchCommon& c, int64_t i0, int64_t n, int smem, cudaStream_t s);
 cudaError_t launch_stage_f64(int stage, const LaunchCommon& c, int64_t i0, int64_t n, int smem, cudaStream_t s);
-cudaError_t launch_gauss_reduce(const void* subs, int nsub, const double* part, double* out, cudaStream_t st);
+cudaError_t launch_gauss_reduce(bool f64, const void* subs, int nsub, const void* part, double* out, cudaStream_t st);
 cudaError_t launch_stage_reg(int stage, int rows, const LaunchCommon& c, int64_t i0, int64_t n, int smem, cudaStream_t s);
 cudaError_t launch_stage_z(int zlen, bool heat, bool stag, const LaunchCommon& c, int64_t i0, int64_t n, int smem, cudaStream_t s);
 bool launch_stage_length(int stage, const LaunchCommon& c, int64_t i0, int64_t n, int smem, cudaStream_t s, cudaError_t* err);
@@ -586,7 +586,16 @@ int psatd_plan_create_tuned(psatd_plan_t* out, const int32_t global_n[3], const 
         // PSATD_PACKED_Z asks for it with mixed lengths and staggered fields too
         // (honoured for an even number of modes per plane)
         p->regB = (flags & PSATD_PACKED_Z) && set && even && !p->heat && (!asked || asked == 6);
-        p->zpass = p->regB || (set && (p->heat || (same && !p->stag)) && (!asked || asked == (p->heat ? kZModesHeat : kZModes)));
+        // a few items leave its blocks (six warps or fewer, 12 warps per SM) with
+        // one round, where the eight warps of a generic block finish an item
+        // sooner: one box of 78 x 77 x 64, 385 items, 80 against 73 us a step; it
+        // takes over from one and a half rounds (eight boxes of 48^3, two
+        // rounds: 25 against 31 us for the stage)
+        int64_t zitems = 0;
+        for (const SubDesc& d : p->desc) zitems += (d.q + kZModes - 1) / kZModes;
+        const bool many = zitems * 2 >= 3 * int64_t(kSms) * (192 / std::max(d0.L[2], 1));
+        p->zpass = p->regB || (set && (p->heat || (same && !p->stag && many)) &&
+                               (!asked || asked == (p->heat ? kZModesHeat : kZModes)));
         p->zlen = same ? d0.L[2] : 0;
         // axes of one compiled length in every box (kSplitX, kSplitY, kLongZ) at
         // their default splits
@@ -781,7 +790,7 @@ int psatd_plan_create_tuned(psatd_plan_t* out, const int32_t global_n[3], const 
     p->off_tw = o; o = align_up(o + size_t(p->n_tw) * 4 * esz, 256);   // hi/lo pairs
     p->off_tab = o; o = align_up(o + size_t(p->n_tab) * esz, 256);
     p->off_tabc = o; o = align_up(o + size_t(std::max<int64_t>(p->n_tabc, 1)) * 2 * esz, 256);
-    p->off_gauss = o; o = align_up(o + size_t(std::max<int64_t>(p->items[1], 1)) * 2 * sizeof(double), 256);
+    p->off_gauss = o; o = align_up(o + (p->diag ? size_t(p->items[1]) * 2 * esz : 0), 256);   // partial sums, plan's precision
     p->off_work = o; o = align_up(o + 8 * sizeof(unsigned long long), 256);
     p->off_spec = o; o = align_up(o + size_t(p->spec_elems) * 2 * esz, 256);
     // descriptors of the global-array <-> arena copies
@@ -1029,7 +1038,7 @@ static LaunchCommon common_at(psatd_plan_s* p, char* base, const psatd_fields* f
         c.eb[0] = f->E[0];
         c.eb[1] = p->heat_src ? const_cast<void*>(f->J[0]) : nullptr;   // never written (nout = 1)
     }
-    c.gauss_part = reinterpret_cast<double*>(base + p->off_gauss);
+    c.gauss_part = base + p->off_gauss;
     c.work = reinterpret_cast<unsigned long long*>(base + p->off_work);
     c.err = reinterpret_cast<unsigned int*>(base + p->off_work + 7 * sizeof(unsigned long long));
     c.persistent = (p->flags & PSATD_GRID_PER_ITEM) ? 0 : 1;
@@ -1140,7 +1149,7 @@ static int launch_push(psatd_plan_s* p, LaunchCommon c, double* gauss_dev, cudaS
     }
     if ((e = mark(3)) != cudaSuccess) return cuda_fail(p, e, "event record");
     if (p->diag && gauss_dev) {
-        e = launch_gauss_reduce(c.subs, c.nsub, c.gauss_part, gauss_dev, s);
+        e = launch_gauss_reduce(p->f64, c.subs, c.nsub, c.gauss_part, gauss_dev, s);
         if (e != cudaSuccess) return cuda_fail(p, e, "gauss reduce launch");
     }
     return PSATD_OK;

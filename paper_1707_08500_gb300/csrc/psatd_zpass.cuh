@@ -400,8 +400,8 @@ __global__ void __launch_bounds__(NW * 32, MINB) k_pass_z(Args<float> a) {
                 float s1 = 0.f, s2 = 0.f;
                 for (int i = 0; i < NW; ++i) s1 += red[i];
                 for (int i = 0; i < NW; ++i) s2 += red[NW + i];
-                a.gauss_part[2 * it] = double(s1);
-                a.gauss_part[2 * it + 1] = double(s2);
+                a.gauss_part[2 * it] = s1;
+                a.gauss_part[2 * it + 1] = s2;
             }
         }
         cur = nx;
@@ -463,8 +463,8 @@ __global__ void __launch_bounds__(kThreads, 4) k_pass_b_flat(Args<float> a) {
         if (nf > 9) {
             block_sum2(g_res, g_rho, red);
             if (threadIdx.x == 0) {
-                a.gauss_part[2 * it] = double(g_res);
-                a.gauss_part[2 * it + 1] = double(g_rho);
+                a.gauss_part[2 * it] = g_res;
+                a.gauss_part[2 * it + 1] = g_rho;
             }
         }
         __syncthreads();

@@ -52,14 +52,17 @@ def _step(P, wl, flags=0):
 @pytest.mark.parametrize("lz", [32, 48, 64, 80, 96])
 @pytest.mark.parametrize("ycuts", [(7,), (8, 5)])
 def test_z_lengths(P, lz, ycuts):
-    _step(P, _wl(ycuts, (lz,)))
+    # few items: the flag, which an even number of modes per plane needs
+    _step(P, _wl(ycuts, (lz,)), P.PSATD_PACKED_Z)
 
 
-@pytest.mark.parametrize("lz", [32, 96])
-def test_odd_modes_per_plane(P, lz):
-    # local x 20 (11 columns), y 13: 143 modes
-    wl = I.custom("zodd", (12, 5, lz - 2 * NG), ((12,), (5,), (lz - 2 * NG,)), NG, 8, fields="wavepacket", precision="f32")
-    assert wl.subs[0].local[1] * (wl.subs[0].local[0] // 2 + 1) % 2 == 1
+# odd numbers of modes per plane (117 x 97 and 63 x 61), enough items for the
+# stage to be chosen without the flag
+@pytest.mark.parametrize("local", [(192, 117, 32), (120, 63, 96)])
+def test_odd_modes_per_plane(P, local):
+    n = tuple(v - 2 * NG for v in local)
+    wl = I.custom("zodd", n, tuple((v,) for v in n), NG, 8, fields="wavepacket", precision="f32")
+    assert local[1] * (local[0] // 2 + 1) % 2 == 1
     _step(P, wl)
 
 
