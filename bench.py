@@ -125,8 +125,9 @@ def stage_bytes(wl, nf: int, esz: int, nout: int = 6):
     return {"A": A, "B": B, "C": C}, local
 
 
-KERNEL_SOURCES = ("psatd_kernels.cuh", "psatd_kernels_f32.cu", "small_dft.cuh", "psatd_internal.h", "psatd_regfft.cuh",
-                  "psatd_regfft_f32.cu")
+KERNEL_SOURCES = ("psatd_kernels.cuh", "psatd_kernels_f32.cu", "small_dft.cuh", "psatd_internal.h",
+                  "psatd_regfft.cuh", "psatd_regfft_f32.cu", "psatd_launch.cuh", "psatd_zpass.cuh",
+                  "psatd_zpass_f32.cu", "psatd_split_f32.cu")
 
 
 def kernels_sha256() -> str:
@@ -136,6 +137,25 @@ def kernels_sha256() -> str:
         with open(os.path.join(ROOT, "paper_1707_08500_gb300", "csrc", f), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()
+
+
+def z_kernel(sol) -> str:
+    """Name of the kernel that runs a solver's z stage (the plan's rule)."""
+    from paper_1707_08500_gb300 import psatd as P
+    lz = {sd.local[2] for sd in sol.wl.subs}
+    heat = bool(sol.flags & P.PSATD_HEAT)
+    tuning = sol.tuning or {}
+    default = not tuning.get("chunk_b") and not tuning.get("f1", (0, 0, 0))[2]
+    if sol.precision == "f32" and not sol.flags & P.PSATD_GENERIC_PLANES:
+        if P.psatd_plane_engine(sol.plan) & 2:
+            return "k_pass_z"
+        items = sum(-(-sd.local[1] * (sd.local[0] // 2 + 1) // 8) for sd in sol.wl.subs)
+        many = len(lz) == 1 and items * 2 >= 3 * 152 * (192 // max(lz))
+        if default and lz <= {32, 48, 64, 80, 96} and (heat or (many and not sol.flags & P.PSATD_STAGGERED)):
+            return "k_pass_z"
+        if lz == {1} and not heat:
+            return "k_pass_b_flat"
+    return "k_pass_b_heat" if heat else "k_pass_b"
 
 
 def _traffic(kernel: str, workload: str):
@@ -278,11 +298,9 @@ def run_ours(args, rank, world, local_rank):
     dom = max(stage_ms, key=stage_ms.get)
     split = P.psatd_push_launches(sol.plan) - (1 if gauss else 0) == 5
     engine = P.psatd_plane_engine(sol.plan)
-    names = ({"A": "k_rows_fwd+k_cols", "B": "k_pass_b", "C": "k_cols+k_rows_inv"} if split
-             else {"A": "k_pass_a_reg", "B": "k_pass_b", "C": "k_pass_c_reg"} if engine & 1
-             else {"A": "k_pass_a", "B": "k_pass_b", "C": "k_pass_c"})
-    if engine & 2:
-        names["B"] = "k_pass_b_reg"
+    names = ({"A": "k_rows_fwd+k_cols", "C": "k_cols+k_rows_inv"} if split
+             else {"A": "k_pass_a_reg", "C": "k_pass_c_reg"} if engine & 1 else {"A": "k_pass_a", "C": "k_pass_c"})
+    names["B"] = z_kernel(sol)
     stages = {st: {"kernel": names[st], "ms": round(stage_ms[st], 3), "alg_bytes": by[st],
                    "gbs": round(by[st] / (stage_ms[st] / 1e3) / 1e9, 1),
                    "frac": round(by[st] / (stage_ms[st] / 1e3) / 1e9 / peak, 4)} for st in "ABC"}
@@ -561,7 +579,7 @@ def time_workload(name, args, dev, peak):
     stage_ms = {st: sum(evs[k][i].elapsed_time(evs[k][i + 1]) for k in range(K)) / K for i, st in enumerate("ABC")}
     by, local = stage_bytes(wl, 10, 4 if prec == "f32" else 8)
     engine = P.psatd_plane_engine(sol.plan)
-    names = {"A": "k_pass_a_reg" if engine & 1 else "k_pass_a", "B": "k_pass_b_reg" if engine & 2 else "k_pass_b",
+    names = {"A": "k_pass_a_reg" if engine & 1 else "k_pass_a", "B": z_kernel(sol),
              "C": "k_pass_c_reg" if engine & 1 else "k_pass_c"}
     stages = {st: {"kernel": names[st], "ms": round(stage_ms[st], 4),
                    "gbs": round(by[st] / (stage_ms[st] / 1e3) / 1e9, 1),
@@ -717,7 +735,7 @@ def run_heat(args, rank, world, local_rank):
     peak, peak_kind = _peaks()
     dom = max(stage_ms, key=stage_ms.get)
     reg = P.psatd_plane_engine(sol.plan) & 1
-    names = {"A": "k_pass_a_reg" if reg else "k_pass_a", "B": "k_pass_b_heat", "C": "k_pass_c_reg" if reg else "k_pass_c"}
+    names = {"A": "k_pass_a_reg" if reg else "k_pass_a", "B": z_kernel(sol), "C": "k_pass_c_reg" if reg else "k_pass_c"}
     achieved = by[dom] / (stage_ms[dom] / 1e3) / 1e9
     valid = wl.valid_cells
     result = {
