@@ -785,13 +785,15 @@ int psatd_plan_create_tuned(psatd_plan_t* out, const int32_t global_n[3], const 
     p->exch_items = ei;
     // --- workspace layout ------------------------------------------------------
     size_t o = 0;
+    // the counters and the error word first, at the same place in every plan: the
+    // static workspace keeps its error word from one plan's push to another's
+    p->off_work = o; o = align_up(o + 8 * sizeof(unsigned long long), 256);
     p->off_desc = o; o = align_up(o + sizeof(SubDesc) * p->desc.size(), 256);
     p->off_seg = o; o = align_up(o + sizeof(Segment) * p->segs.size(), 256);
     p->off_tw = o; o = align_up(o + size_t(p->n_tw) * 4 * esz, 256);   // hi/lo pairs
     p->off_tab = o; o = align_up(o + size_t(p->n_tab) * esz, 256);
     p->off_tabc = o; o = align_up(o + size_t(std::max<int64_t>(p->n_tabc, 1)) * 2 * esz, 256);
     p->off_gauss = o; o = align_up(o + (p->diag ? size_t(p->items[1]) * 2 * esz : 0), 256);   // partial sums, plan's precision
-    p->off_work = o; o = align_up(o + 8 * sizeof(unsigned long long), 256);
     p->off_spec = o; o = align_up(o + size_t(p->spec_elems) * 2 * esz, 256);
     // descriptors of the global-array <-> arena copies
     for (int s = 0; s < nsub; ++s) {
