@@ -38,10 +38,11 @@ constexpr int kRows = 4;   // rows in flight per thread
 // Copy `rows` rows of `cols` elements of VT (one element, or 16 bytes): row y
 // from in + gy ild + gx, to out + y old + x, where gy = wrap(gy0 + y, ny) and
 // gx = wrap(gx0 + x, nx) (a gather passes ranges that do not wrap).  ild, old,
-// gx0 and nx count elements of VT.
+// gx0 and nx count elements of VT.  Ordinary loads: the kernel ahead may still
+// be writing the source when this block starts (see wait_for_previous_launch).
 template <typename VT>
-__device__ __forceinline__ void copy_rows(const VT* __restrict__ in, int64_t ild, int gx0, int nx, int gy0, int ny,
-                                          VT* __restrict__ out, int64_t old, int cols, int rows) {
+__device__ __forceinline__ void copy_rows(const VT* in, int64_t ild, int gx0, int nx, int gy0, int ny, VT* out, int64_t old,
+                                          int cols, int rows) {
     const int ct = min(cols, kIoThreads), rs = kIoThreads / ct;   // columns and rows of one step of the block
     const int y0 = int(threadIdx.x) / ct, x0 = int(threadIdx.x) - y0 * ct;
     if (y0 >= rs) return;
@@ -53,7 +54,7 @@ __device__ __forceinline__ void copy_rows(const VT* __restrict__ in, int64_t ild
             VT v[kRows];
 #pragma unroll
             for (int k = 0; k < kRows; ++k) {
-                if (y + k * rs < rows) v[k] = __ldg(src + int64_t(gy) * ild);
+                if (y + k * rs < rows) v[k] = src[int64_t(gy) * ild];
                 gy += rs;
                 if (gy >= ny) gy = rs <= ny ? gy - ny : gy % ny;
             }

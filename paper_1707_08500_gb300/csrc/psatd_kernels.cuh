@@ -1255,8 +1255,7 @@ __global__ void __launch_bounds__(kThreads) k_exchange(Args<T> a) {
 
 // ---- per-subdomain reduction of the Gauss partial sums ----------------------
 template <typename T>
-static __global__ void k_gauss_reduce(const SubDesc* __restrict__ subs, int nsub, const T* __restrict__ part,
-                               double* __restrict__ out) {
+static __global__ void k_gauss_reduce(const SubDesc* subs, int nsub, const T* part, double* out) {
     wait_for_previous_launch();
     const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int l = threadIdx.x & 31;

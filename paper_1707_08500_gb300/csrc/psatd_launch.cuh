@@ -8,7 +8,12 @@ namespace psatd {
 // one start its blocks as soon as slots free up (launch_dependents), and none
 // reads or writes global memory, the ticket counter included, before the
 // kernels ahead of it have finished and their writes are visible (wait).  Both
-// do nothing in a launch without the attribute.
+// do nothing in a launch without the attribute.  A block is alive while the
+// kernel ahead still writes, so what that kernel may write (fields, spectra,
+// partial sums, global arrays) is not constant for this one: it is read with
+// ordinary loads or asynchronous copies, never through the non-coherent path
+// (__ldg, or const __restrict__ pointers, which allow it).  That path is for
+// what only set-up copies write: descriptors, tables, twiddles.
 __device__ __forceinline__ void wait_for_previous_launch() {
     asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
     asm volatile("griddepcontrol.wait;\n" ::: "memory");

@@ -1,0 +1,72 @@
+"""Launches that overlap at their ends (psatd_launch.cuh): what the kernel ahead
+may still be writing is not read through the non-coherent path, and calls queued
+back to back on one stream give bit for bit what the same calls give with the
+device synchronised after each."""
+import os
+import re
+
+import pytest
+import torch
+
+from paper_1707_08500_gb300 import inputs as I
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_1707_08500_gb300", "csrc")
+
+
+def _function(file, head):
+    """A function's text, from its head to the closing brace in column 0."""
+    text = open(os.path.join(CSRC, file)).read()
+    return text[text.index(head):].split("\n}\n")[0]
+
+
+@pytest.mark.parametrize("file,head,data", [
+    ("psatd_io.cu", "void copy_rows(", ("in", "src")),
+    ("psatd_kernels.cuh", "void k_gauss_reduce(", ("part",)),
+])
+def test_data_of_the_kernel_ahead_is_read_coherently(file, head, data):
+    body = _function(file, head)
+    for name in data:
+        assert not re.search(r"__restrict__\s+%s\b" % name, body), (head, name)
+        assert not re.search(r"__ldg\(\s*&?%s\b" % name, body), (head, name)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("n,ng,precision", [((32, 32), 8, "f32"), ((23, 18), 3, "f32"), ((16, 16), 8, "f64")])
+def test_queued_calls_equal_synchronised_ones(n, ng, precision):
+    """Scatter J and rho, push with the Gauss sums, gather E and B, four times
+    over: brief launches (eight boxes of 48^3 and smaller), all of them
+    overlapped."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1707_08500_gb300 import build
+    build.build()
+    from paper_1707_08500_gb300 import psatd as P
+    cuts = (n, n, n)
+    wl = I.custom("overlap", (sum(n),) * 3, cuts, ng, 8, fields="wavepacket", precision=precision)
+    glob = {k: v.cuda() for k, v in I.global_fields(wl).items()}
+
+    def run(sync):
+        sol = P.Solver(wl, gauss=True)
+        st = torch.cuda.current_stream().cuda_stream
+        src = [glob[k].to(sol.dtype) for k in ("Jx", "Jy", "Jz", "rho")]
+        src = [[t * (k + 1) for t in src] for k in range(4)]
+        out = [[torch.zeros_like(src[0][0]) for _ in I.EB_NAMES] for _ in range(4)]
+        sums = [torch.zeros_like(sol.gauss_out) for _ in range(4)]
+        P.psatd_scatter_global(sol.plan, [glob[k].to(sol.dtype) for k in I.EB_NAMES], [sol.arenas[k] for k in I.EB_NAMES], st)
+        torch.cuda.synchronize()
+        for k in range(4):
+            P.psatd_scatter_global(sol.plan, src[k], [sol.arenas[v] for v in ("Jx", "Jy", "Jz", "rho")], st)
+            if sync:
+                torch.cuda.synchronize()
+            P.psatd_push(sol.plan, sol.fields, sums[k].data_ptr(), st)
+            if sync:
+                torch.cuda.synchronize()
+            P.psatd_gather_global(sol.plan, [sol.arenas[v] for v in I.EB_NAMES], out[k], st)
+            if sync:
+                torch.cuda.synchronize()
+        torch.cuda.synchronize()
+        assert P.psatd_check(sol.plan) == 0
+        return [t for o in out for t in o] + sums
+
+    for a, b in zip(run(False), run(True)):
+        assert torch.equal(a, b)
