@@ -31,7 +31,7 @@ def test_data_of_the_kernel_ahead_is_read_coherently(file, head, data):
 
 
 @pytest.mark.gpu
-@pytest.mark.parametrize("n,ng,precision", [((32, 32), 8, "f32"), ((23, 18), 3, "f32"), ((16, 16), 8, "f64")])
+@pytest.mark.parametrize("n,ng,precision", [((32, 32), 8, "f32"), ((24, 18), 3, "f32"), ((16, 16), 8, "f64")])
 def test_queued_calls_equal_synchronised_ones(n, ng, precision):
     """Scatter J and rho, push with the Gauss sums, gather E and B, four times
     over: brief launches (eight boxes of 48^3 and smaller), all of them
