@@ -1343,10 +1343,22 @@ static cudaError_t launch_shape(const void* fn, int smem, bool persistent, int* 
     return cudaSuccess;
 }
 
+// Largest tile (bytes) of an inverse plane stage whose launch overlaps the z
+// stage's end.  Its blocks are placed in the holes that the z stage's large
+// blocks leave one by one; small tiles fill them, larger ones do not pack, and
+// some SMs then run the stage with fewer blocks.  Steps with the inverse stage
+// not overlapped / overlapped (passes A and B overlapped in both): tiles of
+// 10 KB, one box of 48^3 36.9 / 32.2 us, eight 78.0 / 76.4; 21 KB, two of 72^3
+// 93.5 / 91.0; 26 KB, four of 80^3 183 / 193, eight one by one 595 / 626; 37
+// KB, two of 96^3 138 / 151; 41 KB, one of 104 x 96 x 32 61.9 / 71.1.
+constexpr int kOverlapTile = 24 * 1024;
+
 // One launch of kernel k: persistent (as many CTAs as can be resident, each
-// drawing work items from the ticket counter) or one CTA per item.
+// drawing work items from the ticket counter) or one CTA per item.  inverse: an
+// inverse plane stage (see kOverlapTile).
 template <typename T>
-static cudaError_t launch_kernel(void (*k)(Args<T>), const Args<T>& a, int smem, cudaStream_t st, int threads = kThreads) {
+static cudaError_t launch_kernel(void (*k)(Args<T>), const Args<T>& a, int smem, cudaStream_t st, int threads = kThreads,
+                                 bool inverse = false) {
     int resident = 0;
     cudaError_t e = launch_shape((const void*)k, smem, a.persistent != 0, &resident, threads);
     if (e != cudaSuccess) return e;
@@ -1356,7 +1368,7 @@ static cudaError_t launch_kernel(void (*k)(Args<T>), const Args<T>& a, int smem,
     // launches lose 1-2% to blocks of the next one that are set up early (48
     // uneven boxes 1320 to 1346 us, 64 boxes of 96^3 2483 to 2501)
     const bool brief = a.nitems <= 16 * int64_t(resident > 0 ? resident : 1);
-    return launch_maybe_overlapped(brief, k, grid, threads, smem, st, a);
+    return launch_maybe_overlapped(brief && !(inverse && smem > kOverlapTile), k, grid, threads, smem, st, a);
 }
 
 // Launch stage `stage` (see stage_item) with geometry G; the exchange and the
@@ -1366,11 +1378,11 @@ static cudaError_t launch_geo(int stage, const Args<T>& a, int smem, cudaStream_
     switch (stage) {
         case 0: return launch_kernel<T>(k_pass_a<T, G>, a, smem, st);
         case 1: return launch_kernel<T>(k_pass_b<T, G>, a, smem, st);
-        case 2: return launch_kernel<T>(k_pass_c<T, G>, a, smem, st);
+        case 2: return launch_kernel<T>(k_pass_c<T, G>, a, smem, st, kThreads, true);
         case 4: return launch_kernel<T>(k_rows_fwd<T>, a, smem, st);
         case 5: return launch_kernel<T>(k_cols<T, false>, a, smem, st);
-        case 6: return launch_kernel<T>(k_cols<T, true>, a, smem, st);
-        case 7: return launch_kernel<T>(k_rows_inv<T>, a, smem, st);
+        case 6: return launch_kernel<T>(k_cols<T, true>, a, smem, st, kThreads, true);
+        case 7: return launch_kernel<T>(k_rows_inv<T>, a, smem, st, kThreads, true);
         case 8: return launch_kernel<T>(k_pass_b_heat<T>, a, smem, st);
         default: return launch_kernel<T>(k_exchange<T>, a, 0, st);
     }

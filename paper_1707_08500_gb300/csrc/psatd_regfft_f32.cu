@@ -12,7 +12,7 @@ cudaError_t launch_stage_reg(int stage, int rows, const LaunchCommon& c, int64_t
     // pass A: a thread per row, up to 64 rows or up to 96
     if (stage == 0) return rows <= 64 ? launch_kernel<float>(k_pass_a_reg<64>, a, smem, st, 64)
                                       : launch_kernel<float>(k_pass_a_reg<96>, a, smem, st, 96);
-    if (stage == 2) return launch_kernel<float>(k_pass_c_reg, a, smem, st, kRegThreads);
+    if (stage == 2) return launch_kernel<float>(k_pass_c_reg, a, smem, st, kRegThreads, true);
     return cudaErrorInvalidValue;
 }
 

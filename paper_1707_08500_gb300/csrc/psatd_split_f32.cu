@@ -21,7 +21,7 @@ bool launch_stage_length(int stage, const LaunchCommon& c, int64_t item0, int64_
                          cudaError_t* err) {
     *err = cudaSuccess;
     const Args<float> a = make_args<float>(c, item0, nitems);
-    auto go = [&](auto k) { if (nitems > 0) *err = launch_kernel<float>(k, a, smem, st); };
+    auto go = [&](auto k) { if (nitems > 0) *err = launch_kernel<float>(k, a, smem, st, kThreads, stage >= 6); };
     if (stage == 1) {
         if (c.longZ == 128) go(k_pass_b<float, GeoZ<kLongZ[0].L, kLongZ[0].M>>);
         else if (c.longZ == 192) go(k_pass_b<float, GeoZ<kLongZ[1].L, kLongZ[1].M>>);
