@@ -1,7 +1,8 @@
 """Launches that overlap at their ends (psatd_launch.cuh): what the kernel ahead
 may still be writing is not read through the non-coherent path, and calls queued
 back to back on one stream give bit for bit what the same calls give with the
-device synchronised after each."""
+device synchronised after each.  Yee steps queued back to back are no slower
+than steps that each find the device idle."""
 import os
 import re
 
@@ -70,3 +71,29 @@ def test_queued_calls_equal_synchronised_ones(n, ng, precision):
 
     for a, b in zip(run(False), run(True)):
         assert torch.equal(a, b)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("n", [(128, 128, 64), (96, 96, 96)])
+def test_queued_yee_steps_are_not_slower_than_single_ones(n):
+    """128 and 108 blocks, fewer than SMs: a step whose blocks start early must
+    not find them crowded on some SMs (two to an SM take twice as long)."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1707_08500_gb300 import build, fdtd
+    build.build()
+    s = fdtd.YeeSolver(n, 0.5, precision="f64", device="cuda")
+    a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+
+    def microseconds(steps):
+        a.record()
+        for _ in range(steps):
+            s.step()
+        b.record()
+        torch.cuda.synchronize()
+        return a.elapsed_time(b) * 1e3 / steps
+
+    microseconds(5)
+    single = sorted(microseconds(1) for _ in range(21))[10]
+    queued = sorted(microseconds(20) for _ in range(9))[4]
+    assert queued < 1.2 * single, (queued, single)
