@@ -7,11 +7,12 @@
 // of them in flight: bound by HBM, or by the L2 for the guard cells that a
 // scatter reads again.  A row per warp and one load in flight took 0.73 ms for
 // four fields into and six out of 64 boxes of 96^3 (2.7 TB/s); this takes
-// 0.345 ms (5.7 TB/s).
+// 0.349 ms (5.7 TB/s).
 #include <cuda_runtime.h>
 
 #include <cstdint>
 
+#include "psatd_internal.h"
 #include "psatd_io.h"
 #include "psatd_launch.cuh"
 
@@ -40,10 +41,22 @@ constexpr int kRows = 4;   // rows in flight per thread
 // gx = wrap(gx0 + x, nx) (a gather passes ranges that do not wrap).  ild, old,
 // gx0 and nx count elements of VT.  Ordinary loads: the kernel ahead may still
 // be writing the source when this block starts (see wait_for_previous_launch).
-template <typename VT>
+// WIDE: rows may be wider than half the block; they go in the number of equal
+// parts that keeps most threads at work (one row of 130 would idle half the
+// block, one of 320 give its last 64 elements a step of their own: six FP64
+// arrays of 640 x 64 x 20 gathered in 28.3 us whole, 20.9 in parts, with the
+// device idle before).  In its own kernel: the search costs boxes of 24^3 6%.
+template <bool WIDE, typename VT>
 __device__ __forceinline__ void copy_rows(const VT* in, int64_t ild, int gx0, int nx, int gy0, int ny, VT* out, int64_t old,
                                           int cols, int rows) {
-    const int ct = min(cols, kIoThreads), rs = kIoThreads / ct;   // columns and rows of one step of the block
+    int ct = min(cols, kIoThreads), rs = kIoThreads / ct;   // columns and rows of one step of the block
+    if (WIDE && cols > kIoThreads / 2) {
+        int parts = (cols + ct - 1) / ct;
+        for (int n = parts + 1, end = parts + 6; n <= end; ++n) {
+            const int c = (cols + n - 1) / n, r = kIoThreads / c;
+            if (n * rs < parts * r) { parts = n; ct = c; rs = r; }
+        }
+    }
     const int y0 = int(threadIdx.x) / ct, x0 = int(threadIdx.x) - y0 * ct;
     if (y0 >= rs) return;
     for (int x = x0; x < cols; x += ct) {
@@ -65,7 +78,7 @@ __device__ __forceinline__ void copy_rows(const VT* in, int64_t ild, int gx0, in
     }
 }
 
-template <typename T>
+template <typename T, bool WIDE>
 __global__ void __launch_bounds__(kIoThreads) k_scatter(IoArgs a) {
     wait_for_previous_launch();
     const int64_t item = blockIdx.x;
@@ -83,13 +96,13 @@ __global__ void __launch_bounds__(kIoThreads) k_scatter(IoArgs a) {
     constexpr int V = 16 / int(sizeof(T));
     using V16 = typename Vec16<T>::type;
     if (d.org[0] % V == 0 && a.gn[0] % V == 0 && Lx % V == 0 && aligned16(in) && aligned16(out))
-        copy_rows(reinterpret_cast<const V16*>(in), int64_t(a.gn[0] / V), d.org[0] / V, a.gn[0] / V, d.org[1], a.gn[1],
+        copy_rows<WIDE>(reinterpret_cast<const V16*>(in), int64_t(a.gn[0] / V), d.org[0] / V, a.gn[0] / V, d.org[1], a.gn[1],
                   reinterpret_cast<V16*>(out), int64_t(Lx / V), Lx / V, Ly);
     else
-        copy_rows(in, int64_t(a.gn[0]), d.org[0], a.gn[0], d.org[1], a.gn[1], out, int64_t(Lx), Lx, Ly);
+        copy_rows<WIDE>(in, int64_t(a.gn[0]), d.org[0], a.gn[0], d.org[1], a.gn[1], out, int64_t(Lx), Lx, Ly);
 }
 
-template <typename T>
+template <typename T, bool WIDE>
 __global__ void __launch_bounds__(kIoThreads) k_gather(IoArgs a) {
     wait_for_previous_launch();
     const int64_t item = blockIdx.x;
@@ -104,10 +117,21 @@ __global__ void __launch_bounds__(kIoThreads) k_gather(IoArgs a) {
     constexpr int V = 16 / int(sizeof(T));
     using V16 = typename Vec16<T>::type;
     if (d.n[0] % V == 0 && Lx % V == 0 && a.gn[0] % V == 0 && aligned16(in) && aligned16(out))
-        copy_rows(reinterpret_cast<const V16*>(in), int64_t(Lx / V), 0, d.n[0] / V, 0, d.n[1], reinterpret_cast<V16*>(out),
+        copy_rows<WIDE>(reinterpret_cast<const V16*>(in), int64_t(Lx / V), 0, d.n[0] / V, 0, d.n[1], reinterpret_cast<V16*>(out),
                   int64_t(a.gn[0] / V), d.n[0] / V, d.n[1]);
     else
-        copy_rows(in, int64_t(Lx), 0, d.n[0], 0, d.n[1], out, int64_t(a.gn[0]), d.n[0], d.n[1]);
+        copy_rows<WIDE>(in, int64_t(Lx), 0, d.n[0], 0, d.n[1], out, int64_t(a.gn[0]), d.n[0], d.n[1]);
+}
+
+// Overlapped launches (psatd_launch.cuh) put the early blocks on the SMs that
+// are free first.  A few blocks still get an SM each, and enough of them fill
+// every SM; a number between crowds some SMs while others idle, which costs more
+// than the overlap gains once a block's plane is large: gathers of six arrays,
+// overlapped / not, 520 x 64 x 20 in FP64 (260 KB a plane) 23.9 / 14.5 us, three
+// of 96 x 200 x 64 (150 KB) 14.0 / 10.4, but one of 128 x 128 x 128 in FP32 (36
+// KB a plane) 4.0 / 6.2.
+bool overlap_pays(int64_t blocks, int64_t plane_bytes) {
+    return plane_bytes <= 96 * 1024 || blocks <= kSms / 4 || blocks >= 8 * int64_t(kSms);
 }
 
 }  // namespace
@@ -116,9 +140,13 @@ cudaError_t launch_io(bool scatter, bool f64, const IoArgs& a, cudaStream_t st) 
     const int64_t items = int64_t(a.nfields) * (scatter ? a.planes_local : a.planes_valid);
     if (items <= 0) return cudaSuccess;
     if (items > 2147483647) return cudaErrorInvalidConfiguration;
-    const unsigned grid = unsigned(items);
-    void (*const k)(IoArgs) = scatter ? (f64 ? k_scatter<double> : k_scatter<float>) : (f64 ? k_gather<double> : k_gather<float>);
-    return launch_overlapped(k, dim3(grid), kIoThreads, 0, st, a);
+    const bool wide = a.widest > kIoThreads / 2;
+    auto pick = [&](auto t) -> void (*)(IoArgs) {
+        using T = decltype(t);
+        return scatter ? (wide ? k_scatter<T, true> : k_scatter<T, false>) : (wide ? k_gather<T, true> : k_gather<T, false>);
+    };
+    const bool overlap = overlap_pays(items, a.plane_bytes);
+    return launch_maybe_overlapped(overlap, f64 ? pick(double()) : pick(float()), dim3(unsigned(items)), kIoThreads, 0, st, a);
 }
 
 }  // namespace psatd

@@ -26,6 +26,8 @@ struct IoArgs {
     const int* plane_sub_local;   // subdomain of every local plane (all boxes in order)
     const int* plane_sub_valid;   // subdomain of every valid plane
     int nsub, nfields;
+    int widest;                   // largest local extent along x
+    int64_t plane_bytes;          // largest local plane
     int gn[3];                    // global grid (x, y, z)
     int64_t planes_local, planes_valid;
     const void* in[kIoMaxFields];

@@ -871,6 +871,10 @@ static int io_call(psatd_plan_s* p, bool scatter, const void* const* src, void* 
     a.planes_local = p->io_planes_local;
     a.planes_valid = p->io_planes_valid;
     const size_t esz = p->f64 ? 8 : 4;
+    for (const IoDesc& d : p->io) {
+        a.widest = std::max(a.widest, d.L[0]);
+        a.plane_bytes = std::max(a.plane_bytes, int64_t(esz) * d.L[0] * d.L[1]);
+    }
     for (int f = 0; f < nfields; ++f) {
         if (!src[f] || !dst[f]) return fail(p, PSATD_E_ARG, "null array");
         if (reinterpret_cast<uintptr_t>(src[f]) % esz || reinterpret_cast<uintptr_t>(dst[f]) % esz)

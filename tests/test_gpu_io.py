@@ -26,6 +26,7 @@ CASES = {
     "odd": (((24, 36), (18, 9), (6,)), 3),
     "guards_off_16_bytes": (((24, 40), (16,), (4,)), 6),
     "wide": (((1096,), (3,), (2,)), 2),
+    "rows_of_130_or_260_pieces": (((516,), (9,), (3,)), 2),
     "guards_wider_than_grid": (((4,), (4,), (2,)), 8),
     "one_row": (((32, 32), (1,), (1,)), 0),
 }
