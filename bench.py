@@ -140,22 +140,11 @@ def kernels_sha256() -> str:
 
 
 def z_kernel(sol) -> str:
-    """Name of the kernel that runs a solver's z stage (the plan's rule)."""
+    """Name of the kernel that runs a solver's z stage."""
     from paper_1707_08500_gb300 import psatd as P
-    lz = {sd.local[2] for sd in sol.wl.subs}
-    heat = bool(sol.flags & P.PSATD_HEAT)
-    tuning = sol.tuning or {}
-    default = not tuning.get("chunk_b") and not tuning.get("f1", (0, 0, 0))[2]
-    if sol.precision == "f32" and not sol.flags & P.PSATD_GENERIC_PLANES:
-        if P.psatd_plane_engine(sol.plan) & 2:
-            return "k_pass_z"
-        items = sum(-(-sd.local[1] * (sd.local[0] // 2 + 1) // 8) for sd in sol.wl.subs)
-        many = len(lz) == 1 and items * 2 >= 3 * 152 * (192 // max(lz))
-        if default and lz <= {32, 48, 64, 80, 96} and (heat or (many and not sol.flags & P.PSATD_STAGGERED)):
-            return "k_pass_z"
-        if lz == {1} and not heat:
-            return "k_pass_b_flat"
-    return "k_pass_b_heat" if heat else "k_pass_b"
+    k = P.psatd_stage_kernels(sol.plan)[0]
+    return ("k_pass_z" if k & P.PSATD_KERNEL_Z else "k_pass_b_flat" if k & P.PSATD_KERNEL_Z_FLAT
+            else "k_pass_b_heat" if sol.flags & P.PSATD_HEAT else "k_pass_b")
 
 
 def _traffic(kernel: str, workload: str):
@@ -329,7 +318,8 @@ def run_ours(args, rank, world, local_rank):
         "gpu_launches": args.steps * P.psatd_push_launches(sol.plan),
         "kernels": {"geometry_variant": P.psatd_geometry_variant(sol.plan),
                     "engine": {"planes": "compiled-length" if engine & 1 else "generic",
-                               "z_eq1": "compiled-length" if engine & 2 else "generic"},
+                               "z_eq1": "compiled-length" if P.psatd_stage_kernels(sol.plan)[0] & (
+                                   P.PSATD_KERNEL_Z | P.PSATD_KERNEL_Z_FLAT | P.PSATD_KERNEL_Z_LONG) else "generic"},
                     "tuning": tuning,
                     "persistent": not args.grid_per_item, "cuda_graph_ms_per_step": None if graph_ms is None else round(graph_ms, 4)},
         "clocks": clk.summary(),

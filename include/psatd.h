@@ -328,9 +328,28 @@ int psatd_geometry_variant(psatd_plan_t plan, int32_t* variant);
  * 2 -- PSATD_PACKED_Z is given and honoured: the local z lengths are compiled
  * in (32, 48, 64, 80, 96; default factorisation; chunk_b 0 or 6), every plane
  * has an even number of modes, FP32, not PSATD_HEAT.
- * 0 -- the generic batched kernels throughout.  PSATD_GENERIC_PLANES turns
- * both off. */
+ * 0 -- neither.  PSATD_GENERIC_PLANES turns both off.  The z/Eq. 1 stage has
+ * compiled-length kernels without the flag too: psatd_stage_kernels reports
+ * what runs. */
 int psatd_plane_engine(psatd_plan_t plan, int32_t* engine);
+
+/* Which kernels a push of the plan launches: *kernels receives the bits below
+ * (0: the generic batched kernels throughout), and *chunk_b, unless NULL, the
+ * (ky,kx) modes per work item of the z/Eq. 1 stage (the largest over the
+ * subdomains). */
+#define PSATD_KERNEL_PLANES  0x1  /* plane stages k_pass_a_reg, k_pass_c_reg    */
+#define PSATD_KERNEL_Z       0x2  /* z stage k_pass_z (PSATD_HEAT included)     */
+#define PSATD_KERNEL_Z_FLAT  0x4  /* Eq. 1 alone, k_pass_b_flat: boxes one cell
+                                     deep                                       */
+#define PSATD_KERNEL_Z_LONG  0x8  /* z stage k_pass_b with a long z axis (128,
+                                     192, 256) compiled in                      */
+#define PSATD_KERNEL_SPLIT   0x10 /* split-plane schedule: x rows and y columns
+                                     in separate launches                       */
+#define PSATD_KERNEL_ROWS_X  0x20 /* its row launches with the x length (128,
+                                     192, 256, 384, 512) compiled in            */
+#define PSATD_KERNEL_COLS_Y  0x40 /* its column launches with the y length (128,
+                                     192, 256) compiled in                      */
+int psatd_stage_kernels(psatd_plan_t plan, int32_t* kernels, int32_t* chunk_b);
 
 /* Number of kernel launches one psatd_push enqueues for this plan. */
 int psatd_push_launches(psatd_plan_t plan, int32_t* launches);

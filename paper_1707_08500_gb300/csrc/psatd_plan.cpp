@@ -855,6 +855,22 @@ int psatd_plane_engine(psatd_plan_t p, int32_t* engine) {
     return PSATD_OK;
 }
 
+int psatd_stage_kernels(psatd_plan_t p, int32_t* kernels, int32_t* chunk_b) {
+    if (!p || !kernels) return PSATD_E_ARG;
+    // in the order in which launch_push chooses
+    int k = p->reg ? PSATD_KERNEL_PLANES : 0;
+    if (p->zpass) k |= PSATD_KERNEL_Z;
+    else if (p->flat) k |= PSATD_KERNEL_Z_FLAT;
+    else if (p->longZ) k |= PSATD_KERNEL_Z_LONG;
+    if (p->split) k |= PSATD_KERNEL_SPLIT | (p->splitX ? PSATD_KERNEL_ROWS_X : 0) | (p->splitY ? PSATD_KERNEL_COLS_Y : 0);
+    *kernels = k;
+    if (chunk_b) {
+        *chunk_b = 0;
+        for (const SubDesc& d : p->desc) *chunk_b = std::max(*chunk_b, d.chunkB);
+    }
+    return PSATD_OK;
+}
+
 static int io_call(psatd_plan_s* p, bool scatter, const void* const* src, void* const* dst, int32_t nfields,
                    void* stream) {
     if (!p || !src || !dst) return PSATD_E_ARG;

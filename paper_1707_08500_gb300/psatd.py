@@ -30,6 +30,14 @@ PSATD_HEAT = 0x100
 PSATD_HEAT_SOURCE = 0x200
 PSATD_GENERIC_PLANES = 0x400
 PSATD_PACKED_Z = 0x800
+# bits of psatd_stage_kernels
+PSATD_KERNEL_PLANES = 0x1
+PSATD_KERNEL_Z = 0x2
+PSATD_KERNEL_Z_FLAT = 0x4
+PSATD_KERNEL_Z_LONG = 0x8
+PSATD_KERNEL_SPLIT = 0x10
+PSATD_KERNEL_ROWS_X = 0x20
+PSATD_KERNEL_COLS_Y = 0x40
 
 STATUS = {0: "PSATD_OK", -1: "PSATD_E_ARG", -2: "PSATD_E_SHAPE", -3: "PSATD_E_NOMEM",
           -4: "PSATD_E_CUDA", -5: "PSATD_E_UNSUPPORTED", -6: "PSATD_E_STATE", -7: "PSATD_E_TIMEOUT"}
@@ -39,7 +47,8 @@ EXPORTS = ("psatd_plan", "psatd_plan_create", "psatd_layout", "psatd_arena_elems
            "psatd_destroy", "psatd_status_string", "psatd_last_error", "psatd_push_launches",
            "psatd_push_profiled", "psatd_plan_create_tuned", "psatd_push_static", "psatd_geometry_variant",
            "psatd_yee_step", "psatd_yee_launches", "psatd_check", "psatd_scatter_global",
-           "psatd_gather_global", "psatd_exchange_segments", "psatd_debug_tables", "psatd_plane_engine")
+           "psatd_gather_global", "psatd_exchange_segments", "psatd_debug_tables", "psatd_plane_engine",
+           "psatd_stage_kernels")
 
 STATIC_WORKSPACE_BYTES = 32 * 1024 * 1024
 
@@ -97,6 +106,7 @@ def lib() -> ctypes.CDLL:
         L.psatd_push_launches.argtypes = [P, ctypes.POINTER(I32)]
         L.psatd_geometry_variant.argtypes = [P, ctypes.POINTER(I32)]
         L.psatd_plane_engine.argtypes = [P, ctypes.POINTER(I32)]
+        L.psatd_stage_kernels.argtypes = [P, ctypes.POINTER(I32), ctypes.POINTER(I32)]
         for name in EXPORTS:
             if name not in ("psatd_status_string", "psatd_last_error"):
                 getattr(L, name).restype = ctypes.c_int
@@ -292,6 +302,13 @@ def psatd_plane_engine(plan) -> int:
     n = ctypes.c_int32()
     _check(lib().psatd_plane_engine(plan, ctypes.byref(n)), plan)
     return n.value
+
+
+def psatd_stage_kernels(plan):
+    """(PSATD_KERNEL_* bits of the stages' kernels, modes per z-stage item)."""
+    k, m = ctypes.c_int32(), ctypes.c_int32()
+    _check(lib().psatd_stage_kernels(plan, ctypes.byref(k), ctypes.byref(m)), plan)
+    return k.value, m.value
 
 
 def make_fields(E, B, J, rho=None) -> FieldsT:

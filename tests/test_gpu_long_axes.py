@@ -34,6 +34,11 @@ def test_compiled_axis_lengths(P, local, ng, split):
     wl = I.custom("long", n, tuple((v,) for v in n), ng, 8, fields="wavepacket", precision="f32", c_dt=0.6)
     glob = I.global_fields(wl)
     sol = P.Solver(wl, gauss=True, extra_flags=P.PSATD_SPLIT_PLANES if split else 0)
+    want = P.PSATD_KERNEL_Z_LONG if local[2] >= 128 else 0
+    if split:
+        want |= P.PSATD_KERNEL_SPLIT | (P.PSATD_KERNEL_ROWS_X if local[0] >= 128 else 0) | \
+            (P.PSATD_KERNEL_COLS_Y if local[1] >= 128 else 0)
+    assert P.psatd_stage_kernels(sol.plan)[0] & ~P.PSATD_KERNEL_PLANES == want
     sol.load_global(glob, guards=True)
     sol.push()
     torch.cuda.synchronize()

@@ -38,6 +38,7 @@ def _wl(ycuts, zlens, staggered=False):
 def _step(P, wl, flags=0):
     glob = I.global_fields(wl)
     sol = P.Solver(wl, gauss=True, extra_flags=flags)
+    assert P.psatd_stage_kernels(sol.plan)[0] & (P.PSATD_KERNEL_Z_FLAT if wl.two_d else P.PSATD_KERNEL_Z)
     sol.load_global(glob, guards=True)
     sol.push()
     torch.cuda.synchronize()
@@ -81,6 +82,7 @@ def test_heat(P, zlens, source, ycuts):
     g = I.random_fields(wl.global_n, 3, names=("Jx", "Jy"))
     names = ("T", "S") if source else ("T",)
     hs = P.HeatSolver(wl, 0.4, source=source)
+    assert P.psatd_stage_kernels(hs.plan)[0] & P.PSATD_KERNEL_Z
     hs.load_global({"T": g["Jx"], "S": g["Jy"]}, names=names, guards=True)
     hs.push()
     torch.cuda.synchronize()
