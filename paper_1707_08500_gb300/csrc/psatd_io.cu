@@ -7,7 +7,7 @@
 // of them in flight: bound by HBM, or by the L2 for the guard cells that a
 // scatter reads again.  A row per warp and one load in flight took 0.73 ms for
 // four fields into and six out of 64 boxes of 96^3 (2.7 TB/s); this takes
-// 0.349 ms (5.7 TB/s).
+// 0.336 ms (5.9 TB/s).
 #include <cuda_runtime.h>
 
 #include <cstdint>
@@ -39,8 +39,10 @@ constexpr int kRows = 4;   // rows in flight per thread
 // Copy `rows` rows of `cols` elements of VT (one element, or 16 bytes): row y
 // from in + gy ild + gx, to out + y old + x, where gy = wrap(gy0 + y, ny) and
 // gx = wrap(gx0 + x, nx) (a gather passes ranges that do not wrap).  ild, old,
-// gx0 and nx count elements of VT.  Ordinary loads: the kernel ahead may still
-// be writing the source when this block starts (see wait_for_previous_launch).
+// gx0 and nx count elements of VT.  Loads through the L2 (__ldcg): the kernel
+// ahead may still be writing the source when this block starts (see
+// wait_for_previous_launch), and guard cells are read again by other blocks, not
+// by this one.
 // WIDE: rows may be wider than half the block; they go in the number of equal
 // parts that keeps most threads at work (one row of 130 would idle half the
 // block, one of 320 give its last 64 elements a step of their own: six FP64
@@ -67,7 +69,7 @@ __device__ __forceinline__ void copy_rows(const VT* in, int64_t ild, int gx0, in
             VT v[kRows];
 #pragma unroll
             for (int k = 0; k < kRows; ++k) {
-                if (y + k * rs < rows) v[k] = src[int64_t(gy) * ild];
+                if (y + k * rs < rows) v[k] = __ldcg(src + int64_t(gy) * ild);
                 gy += rs;
                 if (gy >= ny) gy = rs <= ny ? gy - ny : gy % ny;
             }

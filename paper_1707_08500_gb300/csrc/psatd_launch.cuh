@@ -11,7 +11,7 @@ namespace psatd {
 // do nothing in a launch without the attribute.  A block is alive while the
 // kernel ahead still writes, so what that kernel may write (fields, spectra,
 // partial sums, global arrays) is not constant for this one: it is read with
-// ordinary loads or asynchronous copies, never through the non-coherent path
+// ordinary loads, __ldcg, __ldcs or asynchronous copies, never through the non-coherent path
 // (__ldg, or const __restrict__ pointers, which allow it).  That path is for
 // what only set-up copies write: descriptors, tables, twiddles.
 __device__ __forceinline__ void wait_for_previous_launch() {
