@@ -2,8 +2,9 @@
 the split-plane schedule and the z stage of long axes -- against the FP64 oracle:
 every compiled length, row blocks and column blocks with remainders, chunks with
 a ragged end, guards, a length that is not compiled beside one that is.
-Tolerances: one FP32 step, 2e-6 relative L2 (measured 2.6e-7); Gauss sums 1e-3
-(cancellation in i[k].E - rho)."""
+Tolerances: one FP32 step, 2e-6 relative L2 (measured 2.6e-7); Gauss sums 1e-5
+(measured 5.5e-7; squares of i[k].E - rho, whose terms carry the transforms' few
+1e-7)."""
 import numpy as np
 import pytest
 import torch
@@ -46,4 +47,4 @@ def test_compiled_axis_lengths(P, local, ng, split):
     gs = []
     ref = O.step({k: v.numpy() for k, v in glob.items()}, wl, gauss_out=gs)
     assert O.rel_l2({k: v.numpy() for k, v in sol.gather_global().items()}, ref) < 2e-6
-    np.testing.assert_allclose(sol.gauss_sums(), np.array(gs), rtol=1e-3)
+    np.testing.assert_allclose(sol.gauss_sums(), np.array(gs), rtol=1e-5)

@@ -2,8 +2,9 @@
 (psatd_zpass.cuh) against the FP64 oracle: every compiled z length, planes with
 an odd number of modes and a ragged last chunk, the Gauss sums; staggered fields
 and mixed lengths (PSATD_PACKED_Z); the heat equation.  Tolerances: one FP32
-step, 2e-6 relative L2 (measured 2.5e-7); Gauss sums 1e-3 (cancellation in
-i[k].E - rho)."""
+step, 2e-6 relative L2 (measured 2.5e-7); Gauss sums 1e-5 (measured 1.7e-6): a
+sum of squares of i[k].E - rho, whose terms carry the transforms' few 1e-7 of
+|[k]| |E|, here up to twice the residual."""
 import dataclasses
 
 import numpy as np
@@ -46,7 +47,7 @@ def _step(P, wl, flags=0):
     gs = []
     ref = O.step({k: v.numpy() for k, v in glob.items()}, wl, gauss_out=gs)
     assert O.rel_l2({k: v.numpy() for k, v in sol.gather_global().items()}, ref) < 2e-6
-    np.testing.assert_allclose(sol.gauss_sums(), np.array(gs), rtol=1e-3)
+    np.testing.assert_allclose(sol.gauss_sums(), np.array(gs), rtol=1e-5)
 
 
 # local x 22 (12 columns), y 15: 180 modes per plane, 4 in the last chunk of 8
