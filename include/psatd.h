@@ -326,8 +326,8 @@ int psatd_geometry_variant(psatd_plan_t plan, int32_t* variant);
  * lengths compiled in (x: 32, 40, 48, 56, 64, 72, 88, 96, 104; y: 32, 48, 64,
  * 80, 96; default factorisations; not with the split-plane schedule);
  * 2 -- PSATD_PACKED_Z is given and honoured: the local z lengths are compiled
- * in (32, 48, 64, 80, 96; default factorisation; chunk_b 0 or 6), every plane
- * has an even number of modes, FP32, not PSATD_HEAT.
+ * in (32, 48, 64, 80, 96; default factorisation; chunk_b 0, which is 8 modes,
+ * or 6), every plane has an even number of modes, FP32, not PSATD_HEAT.
  * 0 -- neither.  PSATD_GENERIC_PLANES turns both off.  The z/Eq. 1 stage has
  * compiled-length kernels without the flag too: psatd_stage_kernels reports
  * what runs. */

@@ -44,8 +44,9 @@ constexpr int kRegX2[] = {32, 40, 48, 56, 64, 72, 88, 96, 104};
 constexpr int kRegY[] = {32, 48, 64, 80, 96};
 constexpr int reg_pitch(int lxh) { return lxh + ((2 - lxh % 4) + 4) % 4; }
 // FP32 z stage of psatd_zpass.cuh (for the z lengths in kRegY): modes per work
-// item, and of the heat equation's one or two fields.
-constexpr int kZModes = 8, kZModesHeat = 16;
+// item, of the heat equation's one or two fields, and the narrower width that
+// PSATD_PACKED_Z takes when psatd_tuning asks for it.
+constexpr int kZModes = 8, kZModesHeat = 16, kZModesAsked = 6;
 constexpr int kSms = 152;         // SMs of the GPU that the rules on item counts are for
 constexpr int64_t kZMaxElems = int64_t(1) << 31;   // of a box's coefficient tables and of its spectra (32-bit offsets)
 

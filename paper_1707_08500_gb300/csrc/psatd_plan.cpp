@@ -22,7 +22,7 @@ cudaError_t launch_stage_f32(int stage, const LaunchCommon& c, int64_t i0, int64
 cudaError_t launch_stage_f64(int stage, const LaunchCommon& c, int64_t i0, int64_t n, int smem, cudaStream_t s);
 cudaError_t launch_gauss_reduce(bool f64, const void* subs, int nsub, const void* part, double* out, cudaStream_t st);
 cudaError_t launch_stage_reg(int stage, int rows, const LaunchCommon& c, int64_t i0, int64_t n, int smem, cudaStream_t s);
-cudaError_t launch_stage_z(int zlen, bool heat, bool stag, const LaunchCommon& c, int64_t i0, int64_t n, int smem, cudaStream_t s);
+cudaError_t launch_stage_z(int zlen, int modes, bool heat, bool stag, const LaunchCommon& c, int64_t i0, int64_t n, int smem, cudaStream_t s);
 bool launch_stage_length(int stage, const LaunchCommon& c, int64_t i0, int64_t n, int smem, cudaStream_t s, cudaError_t* err);
 cudaError_t launch_stage_flat(bool stag, const LaunchCommon& c, int64_t i0, int64_t n, cudaStream_t s);
 }  // namespace psatd
@@ -585,7 +585,7 @@ int psatd_plan_create_tuned(psatd_plan_t* out, const int32_t global_n[3], const 
         const int asked = tuning ? tuning->chunk_b : 0;
         // PSATD_PACKED_Z asks for it with mixed lengths and staggered fields too
         // (honoured for an even number of modes per plane)
-        p->regB = (flags & PSATD_PACKED_Z) && set && even && !p->heat && (!asked || asked == 6);
+        p->regB = (flags & PSATD_PACKED_Z) && set && even && !p->heat && (!asked || asked == kZModesAsked);
         // a few items leave its blocks (six warps or fewer, 12 warps per SM) with
         // one round, where the eight warps of a generic block finish an item
         // sooner: one box of 78 x 77 x 64, 385 items, 80 against 73 us a step; it
@@ -621,7 +621,7 @@ int psatd_plan_create_tuned(psatd_plan_t* out, const int32_t global_n[3], const 
         if (!(tuning && tuning->chunk_b) && p->heat)       // one or two fields: wider chunks
             while (M < 64 && int64_t(p->nf) * d.L[2] * (2 * M) * csz <= 32 * 1024) M *= 2;
         while (M > 1 && int64_t(p->nf) * (d.L[2] * M + 16) * csz > 200 * 1024) M /= 2;
-        if (p->zpass) M = p->heat ? kZModesHeat : kZModes;
+        if (p->zpass) M = p->heat ? kZModesHeat : p->regB && M == kZModesAsked ? kZModesAsked : kZModes;
         for (const ZChunk& v : kLongZ) if (p->longZ == v.L) M = v.M;
         d.chunkB = M;
         d.lgB = 0;
@@ -1130,7 +1130,7 @@ static int launch_push(psatd_plan_s* p, LaunchCommon c, double* gauss_dev, cudaS
         }
         if (!p->plain && (e = mark(1)) != cudaSuccess) return cuda_fail(p, e, "event record");
         if (p->zpass) {
-            if ((e = launch_stage_z(p->zlen, p->heat, p->stag, c, r.b0, r.bn, p->smemB, s)) != cudaSuccess)
+            if ((e = launch_stage_z(p->zlen, p->desc[0].chunkB, p->heat, p->stag, c, r.b0, r.bn, p->smemB, s)) != cudaSuccess)
                 return cuda_fail(p, e, "pass B launch");
         } else if (p->flat) {
             if ((e = launch_stage_flat(p->stag, c, r.b0, r.bn, s)) != cudaSuccess) return cuda_fail(p, e, "pass B launch");

@@ -3,8 +3,7 @@
 an odd number of modes and a ragged last chunk, the Gauss sums; staggered fields
 and mixed lengths (PSATD_PACKED_Z); the heat equation.  Tolerances: one FP32
 step, 2e-6 relative L2 (measured 2.5e-7); Gauss sums 1e-5 (measured 1.7e-6): a
-sum of squares of i[k].E - rho, whose terms carry the transforms' few 1e-7 of
-|[k]| |E|, here up to twice the residual."""
+sum of squares of i[k].E - rho, whose terms carry the transforms' few 1e-7."""
 import dataclasses
 
 import numpy as np
@@ -36,9 +35,9 @@ def _wl(ycuts, zlens, staggered=False):
     return dataclasses.replace(wl, staggered=staggered)
 
 
-def _step(P, wl, flags=0):
+def _step(P, wl, flags=0, tuning=None):
     glob = I.global_fields(wl)
-    sol = P.Solver(wl, gauss=True, extra_flags=flags)
+    sol = P.Solver(wl, gauss=True, extra_flags=flags, tuning=tuning)
     assert P.psatd_stage_kernels(sol.plan)[0] & (P.PSATD_KERNEL_Z_FLAT if wl.two_d else P.PSATD_KERNEL_Z)
     sol.load_global(glob, guards=True)
     sol.push()
@@ -73,6 +72,18 @@ def test_mixed_lengths_and_stagger(P, zlens, staggered):
     wl = _wl((8,), zlens, staggered)
     assert P.psatd_plane_engine(P.Solver(wl, extra_flags=P.PSATD_PACKED_Z).plan) & 2
     _step(P, wl, P.PSATD_PACKED_Z)
+
+
+# six modes per item asked for: 14 x 11 and 16 x 11 modes per plane, 4 and 2 of
+# them in the last chunk
+@pytest.mark.parametrize("zlens,staggered", [((32,), False), ((96,), False), ((48, 80), False), ((64, 96), True)])
+def test_six_modes_per_item(P, zlens, staggered):
+    zc = tuple(v - 2 * NG for v in zlens)
+    wl = I.custom("z6", (12, 14, sum(zc)), ((12,), (6, 8), zc), NG, 8, fields="wavepacket", c_dt=0.6, precision="f32")
+    wl = dataclasses.replace(wl, staggered=staggered)
+    tuning = {"chunk_b": 6}
+    assert P.psatd_stage_kernels(P.Solver(wl, extra_flags=P.PSATD_PACKED_Z, tuning=tuning).plan) == (P.PSATD_KERNEL_Z, 6)
+    _step(P, wl, P.PSATD_PACKED_Z, tuning)
 
 
 @pytest.mark.parametrize("zlens", [(32,), (48, 64), (80, 96)])

@@ -32,6 +32,10 @@ def test_z_stage(P):
     # one box of 64^3 is too few items for k_pass_z, unless asked for it
     assert boxes(P, 1, (64, 64, 64), F) == (K.PSATD_KERNEL_PLANES, 8)
     assert boxes(P, 1, (64, 64, 64), F | P.PSATD_PACKED_Z) == (K.PSATD_KERNEL_PLANES | K.PSATD_KERNEL_Z, 8)
+    # a chunk width asked for is the one that runs
+    assert boxes(P, 1, (64, 64, 64), F | P.PSATD_PACKED_Z, tuning={"chunk_b": 6}) == (K.PSATD_KERNEL_PLANES | K.PSATD_KERNEL_Z, 6)
+    assert boxes(P, 8, (96, 96, 96), F, tuning={"chunk_b": 8}) == (K.PSATD_KERNEL_PLANES | K.PSATD_KERNEL_Z, 8)
+    assert boxes(P, 8, (96, 96, 96), F, tuning={"chunk_b": 6}) == (K.PSATD_KERNEL_PLANES, 6)
     # not for staggered fields, other lengths or chunks; the heat equation always
     assert boxes(P, 8, (96, 96, 96), F | P.PSATD_STAGGERED)[0] == K.PSATD_KERNEL_PLANES
     assert boxes(P, 8, (96, 96, 88), F)[0] == K.PSATD_KERNEL_PLANES
