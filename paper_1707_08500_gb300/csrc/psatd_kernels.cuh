@@ -61,22 +61,44 @@ template <> struct vec2<double> { using type = double2; };
 template <typename T>
 struct alignas(4 * sizeof(T)) twd { cpx<T> hi, lo; };
 
-// The kernels use the hi part alone, which the host rounds so that each FP32
-// twiddle's magnitude is as close to 1 as neighbouring values allow (the
-// transform then stays closer to unitary; the phase error this trades in
-// cancels between a forward transform and its inverse).  Measured over 100
-// FP32 steps against the FP64 oracle: 5.1e-6, and 3.8e-6 with hi + lo
-// products, at twice their cost.
+// FP32 table twiddles: the hi part alone (PSATD_TW_HILO 0, the default), which
+// the host rounds so that each twiddle's magnitude is as close to 1 as
+// neighbouring values allow (the transform then stays closer to unitary; the
+// phase error this trades in cancels between a forward transform and its
+// inverse), or hi + lo pairs (a build with PSATD_TW_HILO 1: FP64-exact
+// twiddles at twice the products).  Measured over 100 FP32 steps against the
+// FP64 oracle: 5.4e-6 (hi alone) and 4.1e-6 (hi + lo).
+#ifndef PSATD_TW_HILO
+#define PSATD_TW_HILO 0
+#endif
 template <typename T>
-__device__ __forceinline__ cpx<T> ld_tw(const twd<T>* p) {
+using tw_t = typename std::conditional<sizeof(T) == 4 && PSATD_TW_HILO, twd<T>, cpx<T>>::type;   // a loaded twiddle
+template <typename T>
+__device__ __forceinline__ tw_t<T> ld_tw(const twd<T>* p) {
     using V = typename vec2<T>::type;
     const V v = __ldg(reinterpret_cast<const V*>(p));
-    return mk(v.x, v.y);
+    if constexpr (sizeof(T) == 4 && PSATD_TW_HILO) {
+        const V l = __ldg(reinterpret_cast<const V*>(p) + 1);
+        return tw_t<T>{mk(v.x, v.y), mk(l.x, l.y)};
+    } else {
+        return mk(v.x, v.y);
+    }
 }
 template <typename T>   // v * w
 __device__ __forceinline__ cpx<T> mul_tw(cpx<T> v, cpx<T> w) { return cmul(v, w); }
 template <typename T>   // v * conj(w)
 __device__ __forceinline__ cpx<T> mul_tw_conj(cpx<T> v, cpx<T> w) { return cmulc(v, w); }
+// the same with a hi + lo twiddle: the lo products first
+template <typename T>
+__device__ __forceinline__ cpx<T> mul_tw(cpx<T> v, const twd<T>& w) {
+    return mk(fma_t(v.x, w.hi.x, fma_t(-v.y, w.hi.y, fma_t(v.x, w.lo.x, -v.y * w.lo.y))),
+              fma_t(v.x, w.hi.y, fma_t(v.y, w.hi.x, fma_t(v.x, w.lo.y, v.y * w.lo.x))));
+}
+template <typename T>
+__device__ __forceinline__ cpx<T> mul_tw_conj(cpx<T> v, const twd<T>& w) {
+    return mk(fma_t(v.x, w.hi.x, fma_t(v.y, w.hi.y, fma_t(v.x, w.lo.x, v.y * w.lo.y))),
+              fma_t(-v.x, w.hi.y, fma_t(v.y, w.hi.x, fma_t(-v.x, w.lo.y, v.y * w.lo.x))));
+}
 
 template <typename T>
 struct Args {
@@ -252,7 +274,7 @@ __device__ __forceinline__ void dft_runtime(cpx<T>* v, int R, const twd<T>* __re
         for (int r = 1; r < R; ++r) {
             e += k;
             if (e >= R) e -= R;                   // e = r k mod R
-            const cpx<T> w = ld_tw(tw_n + e * nR);
+            const tw_t<T> w = ld_tw(tw_n + e * nR);
             acc = acc + (INV ? mul_tw_conj(v[r], w) : mul_tw(v[r], w));
         }
         out[k] = acc;
@@ -276,7 +298,7 @@ __device__ __forceinline__ void stage_mid(cpx<T>* sm, const Batch& bt, const Axi
         for (int r = 0; r < f2; ++r) v[r] = p[r * es];
         dft_runtime<INV>(v, f2, tw_n, ax.n / f2);
         for (int r = 0; r < f2; ++r) {
-            const cpx<T> w = ld_tw(tw_n + (INV ? (j2 + f3 * r) * k1 : j2 * r * f1));
+            const tw_t<T> w = ld_tw(tw_n + (INV ? (j2 + f3 * r) * k1 : j2 * r * f1));
             p[r * es] = INV ? mul_tw_conj(v[r], w) : mul_tw(v[r], w);
         }
     });
@@ -389,18 +411,18 @@ __device__ __forceinline__ void split_pair_ax(int i, int h, const AxisPlan& ax, 
 // given halved (wh = w/2): 12 operations, the factor 1/2 of e inside the
 // multiply-adds and that of o in wh, both exact.
 template <typename T>
-__device__ __forceinline__ void split_pair_v(cpx<T> A, cpx<T> B, cpx<T> wh, cpx<T>& outA, cpx<T>& outB) {
+__device__ __forceinline__ void split_pair_v(cpx<T> A, cpx<T> B, const tw_t<T>& wh, cpx<T>& outA, cpx<T>& outB) {
     const cpx<T> s = mk(A.x + B.x, A.y - B.y), d = mk(A.x - B.x, A.y + B.y);
-    const cpx<T> wo = cmul(mk(d.y, -d.x), wh);
+    const cpx<T> wo = mul_tw(mk(d.y, -d.x), wh);
     outA = mk(fma_t(T(0.5), s.x, wo.x), fma_t(T(0.5), s.y, wo.y));
     outB = mk(fma_t(T(0.5), s.x, -wo.x), fma_t(T(-0.5), s.y, wo.y));
 }
 // Inverse of split_pair_v: X[pa] = A, X[pb] = B -> Z[pa] = e + i o,
 // Z[pb] = conj(e) + i conj(o), e = A + conj B, o = (A - conj B) conj(w).
 template <typename T>
-__device__ __forceinline__ void merge_pair_v(cpx<T> A, cpx<T> B, cpx<T> wh, cpx<T>& outA, cpx<T>& outB) {
+__device__ __forceinline__ void merge_pair_v(cpx<T> A, cpx<T> B, const tw_t<T>& wh, cpx<T>& outA, cpx<T>& outB) {
     const cpx<T> e = mk(A.x + B.x, A.y - B.y);
-    const cpx<T> o = cmulc(mk(A.x - B.x, A.y + B.y), wh);
+    const cpx<T> o = mul_tw_conj(mk(A.x - B.x, A.y + B.y), wh);
     outA = mk(fma_t(T(-2), o.y, e.x), fma_t(T(2), o.x, e.y));
     outB = mk(fma_t(T(2), o.y, e.x), fma_t(T(2), o.x, -e.y));
 }

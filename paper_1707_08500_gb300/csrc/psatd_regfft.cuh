@@ -335,7 +335,7 @@ __device__ __forceinline__ void col_inv1(const ColPair& cp, int q, int nq, const
         cp.st(k * F2, a[0], b[0]);
 #pragma unroll
         for (int r = 1; r < F2; ++r) {
-            const cpx<float> w = ld_tw(tw + r * k);
+            const tw_t<float> w = ld_tw(tw + r * k);
             cp.st(k * F2 + r, mul_tw_conj(a[r], w), mul_tw_conj(b[r], w));
         }
     }
@@ -393,7 +393,7 @@ __device__ __forceinline__ void cols_fwd1(cpx<float>* sm, int P, int np, const t
         q[np] = b[0];
 #pragma unroll
         for (int r = 1; r < F1; ++r) {
-            const cpx<float> w = ld_tw(tw + j * r);
+            const tw_t<float> w = ld_tw(tw + j * r);
             q[r * st] = mul_tw(a[r], w);
             q[r * st + np] = mul_tw(b[r], w);
         }

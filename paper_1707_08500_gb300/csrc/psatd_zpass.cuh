@@ -189,7 +189,7 @@ __global__ void __launch_bounds__(NW * 32, MINB) k_pass_z(Args<float> a) {
     __shared__ SubDesc s_d[3];             // descriptors of the current item and the next two
     __shared__ int64_t s_it[3];            // their numbers, -1 past the last
     __shared__ float red[2 * NW];
-    __shared__ cpx<float> s_tw[CN ? 4 * CN : 96];   // w^(j r) at j N + r, j < 4, r < N
+    __shared__ tw_t<float> s_tw[CN ? 4 * CN : 96];   // w^(j r) at j N + r, j < 4, r < N
     const int warp = int(threadIdx.x) >> 5, lane = int(threadIdx.x) & 31;
     const TicketDraw<float> draw{a};
     wait_for_previous_launch();
@@ -344,7 +344,7 @@ __global__ void __launch_bounds__(NW * 32, MINB) k_pass_z(Args<float> a) {
                         g_rho = fmaf(wgt, fmaf(rho[i].x, rho[i].x, rho[i].y * rho[i].y), g_rho);
                     }
                 }
-                const cpx<float> w1 = s_tw[N1 + k1], w2 = s_tw[2 * N1 + k1], w3 = s_tw[3 * N1 + k1];
+                const tw_t<float> w1 = s_tw[N1 + k1], w2 = s_tw[2 * N1 + k1], w3 = s_tw[3 * N1 + k1];
 #pragma unroll
                 for (int f = 0; f < 6; ++f) {
                     Dft<4, true>::run(v[f]);
