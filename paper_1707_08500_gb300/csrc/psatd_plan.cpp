@@ -570,8 +570,11 @@ int psatd_plan_create_tuned(psatd_plan_t* out, const int32_t global_n[3], const 
     // FP32: the z stage of psatd_zpass.cuh for z lengths in kRegY at their
     // default split (offsets inside a box in 32 bits) and the default chunk, or
     // that same one asked for: for the heat equation, and for Maxwell plans
-    // whose boxes share one z length and that are not staggered -- with mixed
-    // lengths it takes 528 us against the generic stage's 512 on uneven48.
+    // whose boxes share one z length (mixed lengths: 528 us against the generic
+    // stage's 512 on uneven48) and that are not staggered (one length, run-time
+    // instantiation: 1.22 against 1.29 ms on 64 boxes of 96^3, 35 against 37 us on
+    // eight of 48^3 with the Gauss sums, whose step is no faster; those take it by
+    // PSATD_PACKED_Z).
     if (!p->f64 && !(flags & PSATD_GENERIC_PLANES)) {
         bool set = true, same = true, even = true;
         const SubDesc& d0 = p->desc[0];
@@ -587,12 +590,20 @@ int psatd_plan_create_tuned(psatd_plan_t* out, const int32_t global_n[3], const 
         // (honoured for an even number of modes per plane)
         p->regB = (flags & PSATD_PACKED_Z) && set && even && !p->heat && (!asked || asked == kZModesAsked);
         // a few items leave its blocks (six warps or fewer, 12 warps per SM) with
-        // one round, where the eight warps of a generic block finish an item
-        // sooner: one box of 78 x 77 x 64, 385 items, 80 against 73 us a step; it
-        // takes over from one and a half rounds (eight boxes of 48^3, two
-        // rounds: 25 against 31 us for the stage)
+        // one round, or little more, where the eight warps of a generic block
+        // finish an item sooner: one box of 78 x 77 x 64, 385 items, 80 against
+        // 73 us a step, of 80^3, 410 items, 80 against 65; it takes over from one
+        // and a half rounds (eight boxes of 48^3, two rounds, 23 against 33 us
+        // for the stage; one of 96^3, 86 against 101 us a step).  Counted per
+        // launch, which in the plain schedule holds one box (eight of 80^3: 699
+        // against 623 us).  The heat equation's small items need no such rule:
+        // 0.77 to 1.01 of the generic stage's step from 20 items up (1.07 for
+        // eight boxes of 64^3 with a source).
         int64_t zitems = 0;
-        for (const SubDesc& d : p->desc) zitems += (d.q + kZModes - 1) / kZModes;
+        for (const SubDesc& d : p->desc) {
+            const int64_t box = (d.q + kZModes - 1) / kZModes;
+            zitems = p->plain && zitems ? std::min(zitems, box) : p->plain ? box : zitems + box;
+        }
         const bool many = zitems * 2 >= 3 * int64_t(kSms) * (192 / std::max(d0.L[2], 1));
         p->zpass = p->regB || (set && (p->heat || (same && !p->stag && many)) &&
                                (!asked || asked == (p->heat ? kZModesHeat : kZModes)));

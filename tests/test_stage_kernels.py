@@ -46,6 +46,16 @@ def test_z_stage(P):
     assert boxes(P, 1, (30, 30, 192), F) == (K.PSATD_KERNEL_Z_LONG, 4)
 
 
+def test_few_items_are_counted_per_launch(P):
+    """Eight boxes of 64^3 are enough items for k_pass_z in one launch; in the
+    plain schedule, one launch a box, they are not, while boxes of 96^3 are."""
+    F = P.PSATD_F32
+    for size, flags, z in ((64, 0, True), (64, P.PSATD_PLAIN, False), (80, P.PSATD_PLAIN, False), (96, P.PSATD_PLAIN, True)):
+        k = boxes(P, 8, (size,) * 3, F | flags)[0]
+        assert bool(k & P.PSATD_KERNEL_Z) == z, (size, flags)
+    assert boxes(P, 8, (64,) * 3, F | P.PSATD_PLAIN | P.PSATD_PACKED_Z)[0] & P.PSATD_KERNEL_Z
+
+
 def test_split_planes(P):
     F, K, S = P.PSATD_F32, P, P.PSATD_KERNEL_SPLIT
     assert boxes(P, 1, (256, 256, 256), F, ng=0)[0] == S | K.PSATD_KERNEL_ROWS_X | K.PSATD_KERNEL_COLS_Y | K.PSATD_KERNEL_Z_LONG
