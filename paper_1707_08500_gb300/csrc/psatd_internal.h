@@ -36,13 +36,22 @@ constexpr int ilog2(int v) { return v <= 1 ? 0 : 1 + ilog2(v / 2); }
 
 // FP32 plane stages with thread-private transforms of compile-time length
 // (psatd_regfft.cuh): the local x and y lengths they are compiled for, the
-// CTA size, and the shared-memory row pitch of pass A (complex elements: at
-// least Lx/2+1 and = 2 mod 4, so rows are 16-byte aligned and eight
-// consecutive rows start on distinct 16-byte bank groups).
-constexpr int kRegThreads = 128;
+// threads of pass C and the most rows of pass A (a thread per row), and the
+// shared-memory row pitch of pass A for Lx/2 columns (complex elements, = 2 mod
+// 4, so that rows are 16-byte aligned and eight consecutive rows start on
+// distinct 16-byte bank groups).
+constexpr int kRegThreads = 128, kRegRows = 96;
 constexpr int kRegX2[] = {32, 40, 48, 56, 64, 72, 88, 96, 104};
 constexpr int kRegY[] = {32, 48, 64, 80, 96};
-constexpr int reg_pitch(int lxh) { return lxh + ((2 - lxh % 4) + 4) % 4; }
+constexpr int reg_pitch(int cols) { return cols + ((2 - cols % 4) + 4) % 4; }
+// what the kernels rely on: a thread per row; column pairs (c, c + Lx/4); one
+// lane per column pair in pass C
+constexpr bool reg_lengths_fit() {
+    for (int y : kRegY) if (y > kRegRows) return false;
+    for (int x : kRegX2) if (x % 4 || reg_pitch(x / 2) % 2 || x / 2 + 1 > kRegThreads / 2) return false;
+    return true;
+}
+static_assert(reg_lengths_fit(), "kRegX2 and kRegY against the blocks of psatd_regfft.cuh");
 // FP32 z stage of psatd_zpass.cuh (for the z lengths in kRegY): modes per work
 // item, of the heat equation's one or two fields, and the narrower width that
 // PSATD_PACKED_Z takes when psatd_tuning asks for it.

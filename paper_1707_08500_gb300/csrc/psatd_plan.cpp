@@ -724,15 +724,15 @@ int psatd_plan_create_tuned(psatd_plan_t* out, const int32_t global_n[3], const 
     if (p->smemB > kPlaneSmemMax || (p->split && std::max(p->smemR, p->smemK) > kPlaneSmemMax))
         return bad(PSATD_E_UNSUPPORTED, "a stage's tile does not fit in shared memory");
     // FP32 plane stages with compile-time-length transforms: every local x
-    // and y length compiled in, default factorisations, at most 128 rows and
-    // 64 half-spectrum columns (one thread per row, two per column)
+    // and y length compiled in, default factorisations, at most kRegRows rows
+    // (a thread each) and 64 half-spectrum columns
     if (!p->f64 && !p->split && !(flags & PSATD_GENERIC_PLANES)) {
         auto listed = [](const int* l, int n, int v) { for (int i = 0; i < n; ++i) if (l[i] == v) return true; return false; };
         bool ok = true;
         for (const SubDesc& d : p->desc) {
             ok = ok && listed(kRegX2, int(sizeof(kRegX2) / sizeof(int)), d.L[0]) &&
                  listed(kRegY, int(sizeof(kRegY) / sizeof(int)), d.L[1]) && d.ax.f1 == split_first(d.L[0] / 2) &&
-                 d.ay.f1 == split_first(d.L[1]) && d.lxh <= kRegThreads / 2 && d.L[1] <= kRegThreads;
+                 d.ay.f1 == split_first(d.L[1]) && d.lxh <= kRegThreads / 2 && d.L[1] <= kRegRows;
             p->smemAreg = std::max(p->smemAreg, d.L[1] * reg_pitch(d.L[0] / 2) * 8);
             p->regRows = std::max(p->regRows, d.L[1]);
             p->smemCreg = std::max(p->smemCreg, d.q * 8);
