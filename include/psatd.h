@@ -100,11 +100,11 @@ extern "C" {
 #define PSATD_PACKED_Z       0x800 /* FP32: the z/Eq. 1 stage that holds four z
                                      positions of a mode and all its fields in
                                      registers, wherever the local z lengths
-                                     are compiled in (see psatd_plane_engine).
-                                     Without the flag it runs where it is the
-                                     faster one: the heat equation, and
-                                     unstaggered boxes of one z length that
-                                     are not too few                         */
+                                     are compiled in (see psatd_plane_engine;
+                                     the name is that of an earlier kernel).
+                                     Without the flag it runs for the heat
+                                     equation and for unstaggered boxes of one
+                                     z length that are not too few           */
 #define PSATD_SPLIT_PLANES   0x80 /* split-plane schedule: the x and y transforms
                                      of the forward and inverse plane stages run
                                      as separate row and column launches (five

@@ -1,4 +1,4 @@
-"""Build libpsatd.so in-tree for sm_103a with nvcc (no cmake, two translation
+"""Build libpsatd.so in-tree for sm_103a with nvcc (no cmake, the translation
 units compiled in parallel).  ``python -m paper_1707_08500_gb300.build``."""
 from __future__ import annotations
 

@@ -39,7 +39,7 @@
 #define PSATD_MINB_HEAT 4 // 64 registers; 0.48 ms at 2, 0.37 at 3, 0.33 at 4 on 64 boxes of 96^3
 #endif
 #ifndef PSATD_MINB_ROWS
-#define PSATD_MINB_ROWS 4
+#define PSATD_MINB_ROWS 4 // inverse rows; with their columns 561 us at 2, 498 at 3, 469 at 4, 465 at 5 on one 240^3 box
 #endif
 #ifndef PSATD_MINB_A_FIXED
 #define PSATD_MINB_A_FIXED 6    // compile-time geometry: fewer registers live, one more CTA fits
@@ -788,7 +788,6 @@ k_pass_a(Args<T> a) {
 }
 
 // ---- pass B: z transforms and the Eq. 1 update -----------------------------
-// Sum of v over the CTA (a pairwise tree, in T), returned to thread 0.
 // Block sums of two values at once (warp shuffle trees, then thread 0 adds
 // the warps' partials in order); the results are valid in thread 0 only.
 // The caller synchronises the block before red is written again.
@@ -1388,7 +1387,9 @@ static cudaError_t launch_kernel(void (*k)(Args<T>), const Args<T>& a, int smem,
     if (a.persistent) grid = grid_for(a.nitems < resident ? a.nitems : resident);
     // overlapped ends pay where a launch is a few rounds of its blocks; long
     // launches lose 1-2% to blocks of the next one that are set up early (48
-    // uneven boxes 1320 to 1346 us, 64 boxes of 96^3 2483 to 2501)
+    // uneven boxes 1320 to 1346 us, 64 boxes of 96^3 2483 to 2501, both with
+    // every launch overlapped).  The limit of 16 rounds lies between what gains
+    // (27 boxes of 48^3, up to 11 rounds: even) and these, not finer
     const bool brief = a.nitems <= 16 * int64_t(resident > 0 ? resident : 1);
     return launch_maybe_overlapped(brief && !(inverse && smem > kOverlapTile), k, grid, threads, smem, st, a);
 }

@@ -116,8 +116,8 @@ __device__ __forceinline__ void sts4(cpx<float>* p, cpx<float> a, cpx<float> b) 
 // ---- x: one row per thread -----------------------------------------------------
 // The twiddles come from the plan's pool: tw = exp(-2 pi i m/H), m = 0..H-1
 // (the axis table), wp = exp(-2 pi i k/Lx)/2 for the frequency k at every
-// position of the packed transform (the real-split table); both as FP32
-// hi + lo pairs.  Outer loops run at run time so that the code of one length
+// position of the packed transform (the real-split table); both stored as FP32
+// hi + lo pairs (see ld_tw).  Outer loops run at run time so that the code of one length
 // stays small; the DFT bodies are unrolled.
 
 // Forward real transform of one row: row[0..H) holds z[m] = x[2m] + i x[2m+1]
@@ -495,10 +495,10 @@ __global__ void __launch_bounds__(NT, PSATD_REG_THREADS_SM / NT) k_pass_a_reg(Ar
 // ---- pass C ------------------------------------------------------------------
 // Work item (subdomain, E/B component, valid z plane): the plane's half
 // spectrum (contiguous in the spectra block) is copied to shared memory in
-// one bulk copy (pitch Lx/2+1); two threads per column do the inverse y
-// transform; thread t does the merge and inverse x transform of valid row
-// ng + t; then every thread stores the valid cells to every box that holds
-// them (own box and guard images, Fig. 3 step 3).
+// one bulk copy (pitch Lx/2+1); four or eight groups of lanes per column pair do
+// the inverse y transform; thread t does the merge and inverse x transform of
+// valid row ng + t; then every thread stores the valid cells to every box that
+// holds them (own box and guard images, Fig. 3 step 3).
 __global__ void __launch_bounds__(kRegThreads, PSATD_MINB_REG) k_pass_c_reg(Args<float> a) {
     extern __shared__ __align__(16) unsigned char smraw[];
     cpx<float>* sm = reinterpret_cast<cpx<float>*>(smraw);

@@ -23,9 +23,10 @@ bool launch_stage_length(int stage, const LaunchCommon& c, int64_t item0, int64_
     const Args<float> a = make_args<float>(c, item0, nitems);
     auto go = [&](auto k) { if (nitems > 0) *err = launch_kernel<float>(k, a, smem, st, kThreads, stage >= 6); };
     if (stage == 1) {
-        if (c.longZ == 128) go(k_pass_b<float, GeoZ<kLongZ[0].L, kLongZ[0].M>>);
-        else if (c.longZ == 192) go(k_pass_b<float, GeoZ<kLongZ[1].L, kLongZ[1].M>>);
-        else if (c.longZ == 256) go(k_pass_b<float, GeoZ<kLongZ[2].L, kLongZ[2].M>>);
+        static_assert(sizeof(kLongZ) / sizeof(ZChunk) == 3, "one line per entry of kLongZ");
+        if (c.longZ == kLongZ[0].L) go(k_pass_b<float, GeoZ<kLongZ[0].L, kLongZ[0].M>>);
+        else if (c.longZ == kLongZ[1].L) go(k_pass_b<float, GeoZ<kLongZ[1].L, kLongZ[1].M>>);
+        else if (c.longZ == kLongZ[2].L) go(k_pass_b<float, GeoZ<kLongZ[2].L, kLongZ[2].M>>);
         else return false;
         return true;
     }

@@ -21,27 +21,8 @@ struct alignas(2 * sizeof(T)) cpx {
     T x, y;
 };
 
-// Two FP32 lanes advanced by one packed instruction (FFMA2 / FMUL2 / FADD2 of
-// the sm_100 family): the same operation on two independent data sets, e.g. two
-// columns that share every constant and twiddle.  Measured on this part: a
-// packed instruction takes the pipe for two of its cycles (the same FP32 rate
-// as scalar code) but one issue slot, and negating an operand is free.
-struct __align__(8) P2 {
-    float x, y;   // lane 0, lane 1
-    P2() = default;
-    __host__ __device__ constexpr P2(float a) : x(a), y(a) {}
-    __host__ __device__ constexpr P2(float a, float b) : x(a), y(b) {}
-};
-__device__ __forceinline__ float2 f2of(P2 a) { return make_float2(a.x, a.y); }
-__device__ __forceinline__ P2 p2of(float2 a) { return P2(a.x, a.y); }
 __device__ __forceinline__ float fma_t(float a, float b, float c) { return __fmaf_rn(a, b, c); }
 __device__ __forceinline__ double fma_t(double a, double b, double c) { return __fma_rn(a, b, c); }
-__device__ __forceinline__ P2 fma_t(P2 a, P2 b, P2 c) { return p2of(__ffma2_rn(f2of(a), f2of(b), f2of(c))); }
-__device__ __forceinline__ P2 operator*(P2 a, P2 b) { return p2of(__fmul2_rn(f2of(a), f2of(b))); }
-__device__ __forceinline__ P2 operator-(P2 a) { return P2(-a.x, -a.y); }
-__device__ __forceinline__ P2 operator+(P2 a, P2 b) { return p2of(__fadd2_rn(f2of(a), f2of(b))); }
-__device__ __forceinline__ P2 operator-(P2 a, P2 b) { return p2of(__fadd2_rn(f2of(a), f2of(-b))); }
-__device__ __forceinline__ P2& operator+=(P2& a, P2 b) { a = a + b; return a; }
 
 template <typename T>
 __host__ __device__ __forceinline__ cpx<T> mk(T x, T y) { cpx<T> r; r.x = x; r.y = y; return r; }
@@ -121,18 +102,10 @@ template <typename T>
 struct Split32 {
     static constexpr bool kOn = sizeof(T) == 4 && PSATD_DFT_HILO;
 };
-template <>
-struct Split32<P2> {
-    static constexpr bool kOn = PSATD_DFT_HILO;
-};
 template <typename T>
 constexpr T hi_of(double v) { return T(v); }
 template <typename T>
 constexpr T lo_of(double v) { return T(v - double(T(v))); }
-template <>
-constexpr P2 hi_of<P2>(double v) { return P2(float(v)); }
-template <>
-constexpr P2 lo_of<P2>(double v) { return P2(float(v - double(float(v)))); }
 // Whether the FP32 constant v needs its lo part (+-1/2 and the like do not).
 template <typename T>
 constexpr bool has_lo(double v) { return Split32<T>::kOn && v - double(float(v)) != 0.0; }
