@@ -97,3 +97,60 @@ def test_queued_yee_steps_are_not_slower_than_single_ones(n):
     single = sorted(microseconds(1) for _ in range(21))[10]
     queued = sorted(microseconds(20) for _ in range(9))[4]
     assert queued < 1.2 * single, (queued, single)
+
+
+@pytest.mark.gpu
+def test_captured_with_other_streams_and_copies():
+    """A step captured into a graph between work of other kinds -- copies and
+    memsets on its stream, sources spread on a second stream that joins, a step
+    of another plan that joins -- replays bit for bit as the calls alone."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1707_08500_gb300 import build
+    build.build()
+    from paper_1707_08500_gb300 import psatd as P
+    wl = I.custom("capture", (64,) * 3, ((32, 32),) * 3, 8, 8, fields="wavepacket", precision="f32")
+    glob = {k: v.cuda().float() for k, v in I.global_fields(wl).items()}
+    src = ("Jx", "Jy", "Jz", "rho")
+
+    def fresh():
+        sols = [P.Solver(wl, gauss=True) for _ in range(2)]
+        for s in sols:
+            s.load_global(glob)
+        return sols, [torch.zeros_like(glob["Ex"]) for _ in I.EB_NAMES], [glob[k].clone() for k in src]
+
+    def enqueue(sols, out, up, main, side):
+        a, b = sols
+        up[0].copy_(glob["Jx"])                                        # copies on the main stream
+        a.gauss_out.zero_()
+        side.wait_stream(main)
+        with torch.cuda.stream(side):
+            up[1].copy_(glob["Jy"])
+            P.psatd_scatter_global(a.plan, up, [a.arenas[k] for k in src], side.cuda_stream)
+            b.push(side.cuda_stream)
+        main.wait_stream(side)                                         # joins, then the step
+        a.push(main.cuda_stream)
+        P.psatd_gather_global(a.plan, [a.arenas[k] for k in I.EB_NAMES], out, main.cuda_stream)
+        b.push(main.cuda_stream)
+
+    want, out_w, up_w = fresh()
+    got, out_g, up_g = fresh()
+    main, side = torch.cuda.Stream(), torch.cuda.Stream()
+    torch.cuda.synchronize()
+    with torch.cuda.stream(main):
+        for _ in range(2):
+            enqueue(want, out_w, up_w, main, side)
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=main):
+        enqueue(got, out_g, up_g, torch.cuda.current_stream(), side)
+    for _ in range(2):
+        g.replay()
+    torch.cuda.synchronize()
+    for x, y in zip(out_g, out_w):
+        assert torch.equal(x, y)
+    for s, t in zip(got, want):
+        assert P.psatd_check(s.plan) == 0
+        assert torch.equal(s.gauss_out, t.gauss_out)
+        for k in I.EB_NAMES:
+            assert torch.equal(s.arenas[k], t.arenas[k])
