@@ -334,11 +334,12 @@ int launch(const int32_t n[3], double c_dt, const double dx[3], const psatd_fiel
     auto k = fast ? k_yee<T, true> : k_yee<T, false>;
     if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess)
         return PSATD_E_CUDA;
-    // Overlapped ends pay for a few blocks (32^3 28.0 to 26.1 us); more of them
-    // crowd the SMs that are free first, while others idle (128 x 128 x 64 in
-    // FP64, 128 blocks: 123 to 260 us; 301 x 120 x 77, 450: 56.0 to 62.4)
-    const bool few = int64_t(grid.x) * grid.y * grid.z <= psatd::kSms / 4;
-    return psatd::launch_maybe_overlapped(few, k, grid, NT, smem, st, a) == cudaSuccess ? PSATD_OK : PSATD_E_CUDA;
+    // a few blocks, 32^3: 28.0 us without overlap, 26.1 with it; between, 128 x
+    // 128 x 64 in FP64, 128 blocks: 123 and 260; 301 x 120 x 77, 450: 56.0 and
+    // 62.4; 256 x 256 x 128, 1024: 113.7 and 116.2; many, 320 x 256 x 128, 1280:
+    // 134.4 and 132.8; 768 x 320 x 250, 7680: 693.3 and 691.6
+    const bool overlap = psatd::overlap_pays(int64_t(grid.x) * grid.y * grid.z);
+    return psatd::launch_maybe_overlapped(overlap, k, grid, NT, smem, st, a) == cudaSuccess ? PSATD_OK : PSATD_E_CUDA;
 }
 
 }  // namespace

@@ -125,17 +125,6 @@ __global__ void __launch_bounds__(kIoThreads) k_gather(IoArgs a) {
         copy_rows<WIDE>(in, int64_t(Lx), 0, d.n[0], 0, d.n[1], out, int64_t(a.gn[0]), d.n[0], d.n[1]);
 }
 
-// Overlapped launches (psatd_launch.cuh) put the early blocks on the SMs that
-// are free first.  A few blocks still get an SM each, and enough of them fill
-// every SM; a number between crowds some SMs while others idle, which costs more
-// than the overlap gains once a block's plane is large: gathers of six arrays,
-// overlapped / not, 520 x 64 x 20 in FP64 (260 KB a plane) 23.9 / 14.5 us, three
-// of 96 x 200 x 64 (150 KB) 14.0 / 10.4, but one of 128 x 128 x 128 in FP32 (36
-// KB a plane) 4.0 / 6.2.
-bool overlap_pays(int64_t blocks, int64_t plane_bytes) {
-    return plane_bytes <= 96 * 1024 || blocks <= kSms / 4 || blocks >= 8 * int64_t(kSms);
-}
-
 }  // namespace
 
 cudaError_t launch_io(bool scatter, bool f64, const IoArgs& a, cudaStream_t st) {
@@ -147,7 +136,11 @@ cudaError_t launch_io(bool scatter, bool f64, const IoArgs& a, cudaStream_t st) 
         using T = decltype(t);
         return scatter ? (wide ? k_scatter<T, true> : k_scatter<T, false>) : (wide ? k_gather<T, true> : k_gather<T, false>);
     };
-    const bool overlap = overlap_pays(items, a.plane_bytes);
+    // Crowded SMs (see overlap_pays) cost more than the overlap gains once a
+    // block's plane is large: gathers of six arrays, overlapped / not, 520 x 64 x
+    // 20 in FP64 (260 KB a plane) 23.9 / 14.5 us, three of 96 x 200 x 64 (150 KB)
+    // 14.0 / 10.4, but one of eight boxes of 96^3 in FP32 (36 KB) 4.0 / 6.2.
+    const bool overlap = a.plane_bytes <= 96 * 1024 || overlap_pays(items);
     return launch_maybe_overlapped(overlap, f64 ? pick(double()) : pick(float()), dim3(unsigned(items)), kIoThreads, 0, st, a);
 }
 

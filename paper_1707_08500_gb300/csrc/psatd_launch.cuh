@@ -2,6 +2,8 @@
 // Launches that overlap at their ends.
 #include <cuda_runtime.h>
 
+#include "psatd_internal.h"
+
 namespace psatd {
 
 // Launches of one stream overlap at their ends: every kernel lets the next
@@ -18,6 +20,11 @@ __device__ __forceinline__ void wait_for_previous_launch() {
     asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
     asm volatile("griddepcontrol.wait;\n" ::: "memory");
 }
+
+// Whether a launch of this many blocks gains by overlapping: its early blocks go
+// to the SMs that are free first, so a few still get an SM each and enough of
+// them fill every SM, but a number between crowds some SMs while others idle.
+constexpr bool overlap_pays(int64_t blocks) { return blocks <= kSms / 4 || blocks >= 8 * int64_t(kSms); }
 
 // Launch that may start before the kernels ahead of it on the stream have
 // finished (see wait_for_previous_launch): a push is three to six dependent
