@@ -151,6 +151,7 @@ struct LaunchCommon {
     int64_t per_sub[5];   // items per subdomain of passes A, B, C and of the split schedule's column stages
                           // (forward, inverse) when every subdomain has the same shape, else 0
     int splitX, splitY, longZ;   // axis lengths compiled in (kSplitX, kSplitY, kLongZ), or 0
+    int ztile;            // dynamic shared memory of the z stage's blocks
     int variant;          // index into kFixedF32 / kFixedF64, or -1 for the descriptor-driven kernels
 };
 

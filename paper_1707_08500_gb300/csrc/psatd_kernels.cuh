@@ -121,6 +121,7 @@ struct Args {
     int nout;               // fields written back (6; heat: 1)
     int staggered;
     int own_only;           // pass C writes only the own valid box
+    int ztile;              // dynamic shared memory of the z stage's blocks (read by launch_kernel)
 };
 
 
@@ -1319,6 +1320,7 @@ static Args<T> make_args(const LaunchCommon& c, int64_t item0, int64_t nitems) {
     a.nout = c.nout;
     a.staggered = c.staggered;
     a.own_only = c.own_only;
+    a.ztile = c.ztile;
     return a;
 }
 
@@ -1371,8 +1373,12 @@ static cudaError_t launch_shape(const void* fn, int smem, bool persistent, int* 
 // not overlapped / overlapped (passes A and B overlapped in both): tiles of
 // 10 KB, one box of 48^3 36.9 / 32.2 us, eight 78.0 / 76.4; 21 KB, two of 72^3
 // 93.5 / 91.0; 26 KB, four of 80^3 183 / 193, eight one by one 595 / 626; 37
-// KB, two of 96^3 138 / 151; 41 KB, one of 104 x 96 x 32 61.9 / 71.1.
-constexpr int kOverlapTile = 24 * 1024;
+// KB, two of 96^3 138 / 151; 41 KB, one of 104 x 96 x 32 61.9 / 71.1.  Where an
+// SM holds two blocks at most anyway (78 KB, one of 192 x 100 x 32 93.5 / 83.4;
+// FP64, one of 60^3 364 / 353), for a few blocks, and behind a z stage whose
+// blocks leave no such holes (at most kOverlapZTile bytes: eight 2D boxes of 72 x
+// 96 33.1 / 30.1), overlapping pays again.
+constexpr int kOverlapTile = 24 * 1024, kOverlapZTile = 8 * 1024;
 
 // One launch of kernel k: persistent (as many CTAs as can be resident, each
 // drawing work items from the ticket counter) or one CTA per item.  inverse: an
@@ -1391,7 +1397,9 @@ static cudaError_t launch_kernel(void (*k)(Args<T>), const Args<T>& a, int smem,
     // every launch overlapped).  The limit of 16 rounds lies between what gains
     // (27 boxes of 48^3, up to 11 rounds: even) and these, not finer
     const bool brief = a.nitems <= 16 * int64_t(resident > 0 ? resident : 1);
-    return launch_maybe_overlapped(brief && !(inverse && smem > kOverlapTile), k, grid, threads, smem, st, a);
+    const bool packs = !inverse || smem <= kOverlapTile || a.ztile <= kOverlapZTile || resident <= 2 * kSms ||
+                       a.nitems <= kSms / 4;
+    return launch_maybe_overlapped(brief && packs, k, grid, threads, smem, st, a);
 }
 
 // Launch stage `stage` (see stage_item) with geometry G; the exchange and the

@@ -1085,6 +1085,7 @@ static LaunchCommon common_at(psatd_plan_s* p, char* base, const psatd_fields* f
     c.splitX = p->splitX;
     c.splitY = p->splitY;
     c.longZ = p->longZ;
+    c.ztile = p->flat ? 0 : p->smemB;
     c.variant = p->variant;
     return c;
 }
